@@ -1,7 +1,7 @@
 """Compile the CUDA library in-tree: paper_2002_11710_gb300/_build/libasched.so.
 
-sm_103a only (GB300); four translation units compiled in parallel and linked into
-one shared library, so it builds in under a minute here and on the GPU host alike.
+sm_103a only (GB300); eight translation units compiled in parallel and linked into
+one shared library, so it builds in a minute or two here and on the GPU host alike.
 """
 from __future__ import annotations
 
@@ -11,8 +11,10 @@ import sys
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
-SRCS = [os.path.join(PKG, "csrc", n) for n in ("asched.cu", "sweep.cu", "matrix.cu", "peaks.cu")]
-HDR = os.path.join(ROOT, "include", "asched.h")
+SRCS = [os.path.join(PKG, "csrc", n) for n in ("carry.cu", "batch.cu", "serving.cu", "full.cu", "sweep.cu", "matrix.cu",
+                                                "asched.cu", "peaks.cu")]
+HDRS = [os.path.join(ROOT, "include", "asched.h")] + [os.path.join(PKG, "csrc", n) for n in (
+    "nvtx_range.h", "kernels.h", "search.cuh", "carry.cuh", "instance.cuh")]
 OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT_DIR, "libasched.so")
 
@@ -32,7 +34,7 @@ def nvcc() -> str:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
-    newest = max(os.path.getmtime(x) for x in SRCS + [HDR, os.path.join(PKG, "csrc", "nvtx_range.h")])
+    newest = max(os.path.getmtime(x) for x in SRCS + HDRS)
     stale = not os.path.exists(LIB) or os.path.getmtime(LIB) < newest
     if force or stale:
         tag = f".tmp{os.getpid()}"
