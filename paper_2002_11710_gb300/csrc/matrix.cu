@@ -25,11 +25,17 @@
 //              at 2e-6 t + (60 / speed) 2^-20 S + 1e-6, S the instance's largest |x| + |y|;
 //   Haversine  angles staged as float pairs hi + lo (lo = float(v - hi)), so a difference
 //              (hi_i - hi_j) + (lo_i - lo_j) is within 2 * 2^-24 of itself plus 2^-47 of
-//              the magnitudes; half-angle differences, sinf (2 ulp), squares, cos(phi)
-//              staged from float64, sum, square root and asinf (2 ulp) with its condition
-//              number below 1.9 for sqrt(a) <= 0.9 (larger values go to float64 outright)
-//              add below 1.8e-6 relative; screened at 8e-6 t + (60 / speed) 2 r 2^-40
-//              (sum of |angles|) + 1e-5.
+//              the magnitudes. Small instances: half-angle differences, sinf (2 ulp),
+//              squares, cos(phi) staged from float64, sum, square root and asinf (2 ulp)
+//              with its condition number below 1.9 for sqrt(a) <= 0.9 (larger values go to
+//              float64 outright) add below 1.8e-6 relative; screened at
+//              8e-6 t + (60 / speed) 2 r 2^-40 (sum of |angles|) + 1e-5. Tiles: longitudes
+//              more than half a turn apart first take the short way round, so that the
+//              sine's condition number stays below 1; own fits of sine (4 * 2^-24) and
+//              arcsine (asinf where sqrt(a) > 1/2) and cos(phi) within 6 * 2^-24 give
+//              27 * 2^-24 for a and below 2.5e-6 for the time (largest found against
+//              80-bit floats over 14 million pairs, poles and date line among them:
+//              8.8e-7, 0.22 of the screen); screened at 4e-6 t + the same rest.
 // Times of 2^22 minutes or more also go to float64 (small instances: every entry of an
 // instance whose largest possible time, 2 S * 60 / speed or pi r * 60 / speed, is not
 // below 2^22, through an infinite tolerance). The float32 time is rounded by adding
@@ -39,28 +45,25 @@
 // the distance to the nearest half minute without a conversion instruction. The float64
 // path is the expression above, on the original float64 coordinates. Lanes that need it
 // queue (row, column, type) in shared memory, so float64 work runs on full warps and
-// follows the number of such entries: large instances keep a queue per warp, drained when
-// it fills and at the end of the instance; small instances one queue per CTA, drained
-// after the pairs by as many warps as it has entries (one, as a rule), entries beyond its
-// capacity computed where they arise.
+// follows the number of such entries: small instances one queue per instance, drained
+// after the pairs by as many warps as it has entries (one, as a rule); tiles one queue over
+// a CTA's whole run. Entries beyond a queue's capacity are computed where they arise.
 //
-// One CTA per instance (grid-stride over instances); the instance's coordinates are
-// staged once in shared memory (angles in radians and cos(phi) for Haversine). Two
-// kernels share a batch, each skipping the other's instances:
+// Both distances are symmetric in every rounded operation (x_i - x_j = -(x_j - x_i)
+// exactly, products commute), so each unordered pair is evaluated once and written to
+// (i, j) and (j, i). Two kernels share a batch:
 //   Small instances (n_types * L^2 + 3 <= kOut words, L <= kSmallLoc: L <= 55 for two
-//   types, 78 for one) are built whole in shared memory by 128-thread CTAs, eight per SM.
-//   Both distances are symmetric in every rounded operation (x_i - x_j = -(x_j - x_i)
-//   exactly, products commute), so each unordered pair i <= j is evaluated once and
-//   written to (i, j) and (j, i). The L (L + 1) / 2 pairs are numbered row by row with row
+//   types, 78 for one), where a batch has enough of them to fill the chip (4 per SM; fewer
+//   join the tiles), are built whole in shared memory by 128-thread CTAs, eight per SM, one
+//   CTA per instance (grid-stride), with its coordinates staged once.
+//   The L (L + 1) / 2 pairs are numbered row by row with row
 //   i folded onto row L - 1 - i (L + 1 pairs per folded row), so the threads take
 //   consecutive numbers with no idle lanes at row ends. The finished matrices, contiguous
 //   in the output, leave by one bulk copy (cp.async.bulk, shared to global) on their
 //   16-byte aligned middle and plain stores on the at most 3 + 3 words around it; the
 //   next instance is staged while that copy runs and waits only for its reads of shared
 //   memory, before its first write of the matrix.
-//   Larger instances: 256-thread CTAs, warps take rows, lanes take columns, so a row's
-//   writes are contiguous. An instance with more locations than the stage holds goes
-//   through float64 alone.
+//   Other instances by tiles of 64 x 64 pairs (travel_tiles_kernel).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stddef.h>
@@ -71,10 +74,10 @@
 
 namespace {
 
-constexpr int kStageLocations = 2048;  // large instances: 5 floats per location, 40 KB of shared memory
-constexpr int kWarps = 8;              // large-instance CTAs: 8 warps, 4 per SM
+constexpr int kWarps = 8;              // tile CTAs: 8 warps, 4 per SM
+constexpr int kTile = 64;              // locations of a tile's side
 constexpr int kThreads = kWarps * 32;
-constexpr int kQueue = 128;            // deferred float64 entries per warp (large instances)
+constexpr int kTileQueue = 512;        // deferred float64 entries per CTA (tiles)
 constexpr int kSmallThreads = 128;     // small-instance CTAs: 4 warps, 8 per SM
 constexpr int kSmallLoc = 80;          // locations of an instance built in shared memory
 constexpr int kOut = 6144;             // int32 words of that instance's matrices
@@ -95,11 +98,6 @@ struct MParams {
   const double* coords;
   int32_t* travel;
   int32_t* status;
-};
-
-struct Stage {  // structure of arrays: hi and lo of both coordinates, cos(phi)
-  float xh[kStageLocations], xl[kStageLocations], yh[kStageLocations], yl[kStageLocations];
-  float cphi[kStageLocations];
 };
 
 struct SmallStage {  // 26,816 bytes: with the queue, eight CTAs fit one SM
@@ -149,34 +147,14 @@ __device__ __forceinline__ int32_t checked(double m, int& bad) {
   return ok ? static_cast<int32_t>(m) : 0;
 }
 
-// One float32 time t32 >= 0 (or NaN): its integer in v, and whether that integer is
-// certain, i.e. t32 < 2^22 lies farther than tol = rel t32 + c from every half minute.
-__device__ __forceinline__ bool round_screened(float t32, float rel, float c, int32_t& v) {
-  const float s = __fadd_rn(t32, 12582912.0f);  // 1.5 * 2^23: rounds t32 half to even
-  const float gap = __fsub_rn(0.5f, fabsf(__fsub_rn(t32, __fsub_rn(s, 12582912.0f))));
-  v = __float_as_int(s) - 0x4B400000;
-  return t32 < 4194304.0f && gap > __fmaf_rn(rel, t32, c);
-}
-
-// The same where t32 < 2^22 is known or rel is infinite (every comparison then fails).
+// One float32 time t32 >= 0 (or NaN): its integer in v, and whether that integer is certain,
+// i.e. t32 lies farther than tol = rel t32 + c from every half minute. t32 < 2^22, or rel is
+// infinite (the comparison then fails).
 __device__ __forceinline__ bool round_screened_bounded(float t32, float rel, float c, int32_t& v) {
   const float s = __fadd_rn(t32, 12582912.0f);
   const float gap = __fsub_rn(0.5f, fabsf(__fsub_rn(t32, __fsub_rn(s, 12582912.0f))));
   v = __float_as_int(s) - 0x4B400000;
   return gap > __fmaf_rn(rel, t32, c);
-}
-
-// Drain a warp's queue of deferred entries into the output rows: each lane takes entries
-// and writes the float64 result.
-__device__ __forceinline__ void drain(const MParams& P, const double* c, int32_t* base, int L, int64_t LL,
-                                      const int* q, int n, int lane, int& bad) {
-  __syncwarp();
-  for (int k = lane; k < n; k += 32) {
-    const int e = q[k];
-    const int i = e >> 12, j = (e >> 1) & 2047, t = e & 1;
-    base[t * LL + static_cast<int64_t>(i) * L + j] = checked(minutes64(P, c, nullptr, i, j, t), bad);
-  }
-  __syncwarp();
 }
 
 // One deferred entry of a small instance: the pair (i, j), i <= j, of type t goes to both
@@ -357,102 +335,249 @@ __global__ void __launch_bounds__(kSmallThreads, 8) travel_small_kernel(const __
   if (bad && P.status) atomicExch(P.status, ASCHED_E_INVALID);
 }
 
-// Instances that are not small: warps take rows, lanes take columns.
-template <bool HAV>
-__global__ void __launch_bounds__(kThreads, 4) travel_kernel(const __grid_constant__ MParams P) {
-  __shared__ Stage st;
-  __shared__ int queue[kWarps][kQueue];
-  __shared__ unsigned s_mag;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float two_r32 = static_cast<float>(P.two_r);
+// ------------------------------------------------------------------ tiles
+
+// Tiles of an instance: the pairs I <= J of blocks of kTile locations.
+__host__ __device__ __forceinline__ int64_t tiles_of(int L, int nt, bool skip_small) {
+  const int64_t n = (static_cast<int64_t>(L) + kTile - 1) / kTile;
+  return skip_small && is_small(L, nt) ? 0 : n * (n + 1) / 2;
+}
+
+// sin(x) for |x| <= pi / 2 (1 + 2^-12): x (1 + x^2 q(x^2)), q fitted for least relative error
+// (6.1e-9) by Lawson's reweighted least squares. Its float32 value is within 3.6 * 2^-24.
+__device__ __forceinline__ float sin_half(float x) {
+  const float z = __fmul_rn(x, x);
+  float q = __fmaf_rn(2.605750296424958e-06f, z, -1.980959059437737e-04f);
+  q = __fmaf_rn(q, z, 8.33306647837162e-03f);
+  q = __fmaf_rn(q, z, -1.6666659712791443e-01f);
+  return __fmaf_rn(__fmul_rn(x, z), q, x);
+}
+
+// asin(sqrt(h)) for 0 <= h <= 1 / 4: r (1 + h q(h)) with r = sqrt(h), q as above (4.9e-9).
+__device__ __forceinline__ float asin_root(float r, float h) {
+  float q = __fmaf_rn(4.216628521680832e-02f, h, 2.4179525673389435e-02f);
+  q = __fmaf_rn(q, h, 4.547037556767464e-02f);
+  q = __fmaf_rn(q, h, 7.495297491550446e-02f);
+  q = __fmaf_rn(q, h, 1.6666752099990845e-01f);
+  return __fmaf_rn(__fmul_rn(r, h), q, r);
+}
+
+struct Deferred {  // an entry left to float64: pair (i, j) of instance b, type t
+  int b, i, j, t;
+};
+
+__device__ __forceinline__ int32_t deferred_value(const MParams& P, const Deferred& e, int& bad) {
+  const double* c = P.coords + 2 * static_cast<int64_t>(P.loc_off[e.b]);
+  return checked(minutes64(P, c, nullptr, e.i, e.j, e.t), bad);
+}
+
+// Instances by tiles of 64 x 64 location pairs, every unordered pair evaluated once: the
+// row block's entries go straight to global memory, the mirrored ones through shared
+// memory, so that both leave by rows. Each CTA takes an equal run of consecutive tiles of
+// all instances together (`tiles` of them), which it finds by a prefix sum over the
+// instances; entries that float32 leaves open wait in a queue over the CTA's whole run, so
+// that float64 works on full warps. Bound by float32 issue (about 60 instructions a
+// Haversine pair) and by the float64 of the open entries. With one CTA per instance the
+// largest instance's CTA set the time: 96 Haversine instances of 40 to 1,000 locations
+// 2,364 us; by tiles, without library sines and arcsines and without float64 cosines per
+// location, 56 us (60 MB written).
+template <bool HAV, int NT>
+__global__ void __launch_bounds__(kThreads, 4) travel_tiles_kernel(const __grid_constant__ MParams P, bool skip_small,
+                                                                   int64_t tiles) {
+  __shared__ float4 hl[2 * kTile];  // (x hi, y hi, x lo, y lo) of the row block, then of the column block
+  __shared__ float cphi[2 * kTile];
+  __shared__ int32_t mirror[NT][kTile][kTile + 1];
+  __shared__ Deferred queue[kTileQueue];
+  __shared__ unsigned s_mag[2], s_qn;
+  __shared__ int s_b;
+  __shared__ int64_t s_sum[kWarps], s_at;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float k0 = P.k32[0], k1 = P.k32[1];
-  const int nt = P.nt;
+  const float two_r32 = static_cast<float>(P.two_r);
+  int64_t t0 = tiles * blockIdx.x / gridDim.x;
+  const int64_t t1 = tiles * (blockIdx.x + 1) / gridDim.x;
   int bad = 0;
-  for (int b = blockIdx.x; b < P.B; b += gridDim.x) {
-    const int lo = P.loc_off[b];
-    const int L = P.loc_off[b + 1] - lo;
-    if (is_small(L, nt)) continue;
-    const double* c = P.coords + 2 * static_cast<int64_t>(lo);
-    int32_t* base = P.travel + P.travel_off[b];
-    const int64_t LL = static_cast<int64_t>(L) * L;
-    if (L > kStageLocations) {  // float64 only
-      for (int i = warp; i < L; i += kWarps)
-        for (int j = lane; j < L; j += 32)
-          for (int t = 0; t < P.nt; ++t)
-            base[t * LL + static_cast<int64_t>(i) * L + j] = checked(minutes64(P, c, nullptr, i, j, t), bad);
-      continue;
+  {  // the instance that holds tile t0: every thread sums a run of instances, then a prefix over threads
+    const int per = (P.B + kThreads - 1) / kThreads;
+    const int b0 = min(tid * per, P.B), b1 = min(b0 + per, P.B);
+    int64_t mine = 0;
+    for (int b = b0; b < b1; ++b) mine += tiles_of(P.loc_off[b + 1] - P.loc_off[b], NT, skip_small);
+    int64_t upto = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t v = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane >= o) upto += v;
     }
-    __syncthreads();  // the previous instance's stage is no longer read
-    if (threadIdx.x == 0) s_mag = 0u;
+    if (lane == 31) s_sum[warp] = upto;
+    if (tid < 2) s_mag[tid] = 0u;
+    if (tid == 0) s_qn = 0u;
     __syncthreads();
-    for (int l = threadIdx.x; l < L; l += blockDim.x) {
-      double x = c[2 * l], y = c[2 * l + 1];
-      const float xh = static_cast<float>(HAV ? x * P.deg : x), yh = static_cast<float>(HAV ? y * P.deg : y);
-      st.xh[l] = xh;
-      st.yh[l] = yh;
-      if (HAV) {
-        x *= P.deg;
-        y *= P.deg;
-        st.cphi[l] = static_cast<float>(cos(x));
-        st.xl[l] = static_cast<float>(x - static_cast<double>(xh));
-        st.yl[l] = static_cast<float>(y - static_cast<double>(yh));
-      } else {
-        const float m = fabsf(xh) + fabsf(yh);  // >= 0 (or NaN, whose bits exceed every finite value)
-        atomicMax(&s_mag, __float_as_uint(m));
+    for (int w = 0; w < warp; ++w) upto += s_sum[w];
+    int64_t at = upto - mine;
+    if (t0 < t1 && at <= t0 && t0 < upto) {  // one thread
+      int b = b0;
+      while (true) {
+        const int64_t n = tiles_of(P.loc_off[b + 1] - P.loc_off[b], NT, skip_small);
+        if (t0 < at + n) break;
+        at += n;
+        ++b;
       }
+      s_b = b;
+      s_at = at;
     }
     __syncthreads();
-    const float S = __uint_as_float(s_mag);
-    int* q = queue[warp];
-    int n = 0;  // queued entries (warp-uniform)
-    for (int i = warp; i < L; i += kWarps) {
-      int32_t* row = base + static_cast<int64_t>(i) * L;
-      int32_t* row1 = row + LL;  // the same row of the second type's matrix
-      for (int j0 = 0; j0 < L; j0 += 32) {
-        const int j = j0 + lane;
-        const bool live = j < L;
-        const int jj = live ? j : i;
-        float d32, rel, abs_part, magk;
+  }
+  if (t0 >= t1) return;
+  int b = s_b, par = 0;
+  int64_t at = s_at;  // tiles before instance b
+  for (int64_t t = t0; t < t1; ++t, par ^= 1) {
+    int lo = P.loc_off[b], L = P.loc_off[b + 1] - lo;
+    int64_t n = tiles_of(L, NT, skip_small);
+    while (t >= at + n) {
+      at += n;
+      ++b;
+      lo = P.loc_off[b];
+      L = P.loc_off[b + 1] - lo;
+      n = tiles_of(L, NT, skip_small);
+    }
+    const double* c = P.coords + 2 * static_cast<int64_t>(lo);
+    int32_t* const base = P.travel + P.travel_off[b];
+    const int64_t LL = static_cast<int64_t>(L) * L;
+    // tile q is (I, J) with q = J (J + 1) / 2 + I
+    const int64_t q = t - at;
+    int J = static_cast<int>((sqrt(static_cast<float>(8 * q + 1)) - 1.0f) * 0.5f);
+    while (static_cast<int64_t>(J) * (J + 1) / 2 > q) --J;
+    while (static_cast<int64_t>(J + 1) * (J + 2) / 2 <= q) ++J;
+    const int I = static_cast<int>(q - static_cast<int64_t>(J) * (J + 1) / 2);
+    const int i0 = I * kTile, j0 = J * kTile;
+    if (tid < 2 * kTile) {  // locations past the end repeat the last one; their entries are not written
+      const int l = min((tid < kTile ? i0 : j0 - kTile) + tid, L - 1);
+      double x = c[2 * l], y = c[2 * l + 1];
+      if (HAV) {
+        x = __dmul_rn(x, P.deg);
+        y = __dmul_rn(y, P.deg);
+      }
+      const float xh = static_cast<float>(x), yh = static_cast<float>(y);
+      float xl = 0.0f, yl = 0.0f;
+      if (HAV) {
+        xl = static_cast<float>(x - static_cast<double>(xh));
+        yl = static_cast<float>(y - static_cast<double>(yh));
+        cphi[tid] = __fmaf_rn(-xl, sinf(xh), cosf(xh));
+      }
+      hl[tid] = make_float4(xh, yh, xl, yl);
+      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(xh) + fabsf(yh)));  // a NaN's bits are largest
+      if (lane == 0) atomicMax(&s_mag[par], m);
+    }
+    if (tid == 0) s_mag[par ^ 1] = 0u;
+    __syncthreads();
+    const float S = __uint_as_float(s_mag[par]);  // the largest |x| + |y| of the tile's locations
+    float c0, c1, rel;
+    if (HAV) {
+      const float magk = two_r32 * 9.094947e-13f * 2.0f * S;  // 2 r 2^-40 (sum of |angles|)
+      c0 = __fmaf_rn(k0, magk, 1e-5f);
+      c1 = __fmaf_rn(k1, magk, 1e-5f);
+      rel = P.rel_hav * 0.5f;
+    } else {
+      const float magk = 9.536743e-7f * S;  // 2^-20 S
+      c0 = __fmaf_rn(k0, magk, 1e-6f);
+      c1 = __fmaf_rn(k1, magk, 1e-6f);
+      // every time is below 2 S k (1 + 10 2^-24); false for a NaN or infinite S
+      rel = 2.0f * S * fmaxf(k0, NT > 1 ? k1 : 0.0f) * 1.001f < 4194304.0f ? 2e-6f : __int_as_float(0x7f800000);
+    }
+    const bool diagonal = I == J;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int jl = lane + 32 * h, j = j0 + jl;
+      if (j0 + 32 * h >= L) break;
+      const bool live = j < L;
+      const float4 bb = hl[kTile + jl];
+      const float cj = HAV ? cphi[kTile + jl] : 0.0f;
+      const int rows = min(kTile, L - i0);
+      int32_t* out = base + static_cast<int64_t>(i0 + warp) * L + j;
+      for (int il = warp; il < rows; il += kWarps, out += static_cast<int64_t>(kWarps) * L) {
+        const float4 a = hl[il];
+        float d32;
         bool screen = true;
         if (HAV) {
-          const float dx = __fadd_rn(__fsub_rn(st.xh[i], st.xh[jj]), __fsub_rn(st.xl[i], st.xl[jj]));
-          const float dy = __fadd_rn(__fsub_rn(st.yh[i], st.yh[jj]), __fsub_rn(st.yl[i], st.yl[jj]));
-          const float s1 = sinf(__fmul_rn(dx, 0.5f)), s2 = sinf(__fmul_rn(dy, 0.5f));
-          const float a = __fadd_rn(__fmul_rn(s1, s1), __fmul_rn(__fmul_rn(st.cphi[i], st.cphi[jj]), __fmul_rn(s2, s2)));
-          const float r = __fsqrt_rn(a);
-          screen = r <= 0.9f;
-          d32 = __fmul_rn(two_r32, asinf(r));
-          rel = 8e-6f;
-          abs_part = 1e-5f;
-          magk = two_r32 * 9.094947e-13f *  // 2 r 2^-40 (sum of |angles|)
-                 (fabsf(st.xh[i]) + fabsf(st.xh[jj]) + fabsf(st.yh[i]) + fabsf(st.yh[jj]));
-        } else {
-          const float dx = __fsub_rn(st.xh[i], st.xh[jj]), dy = __fsub_rn(st.yh[i], st.yh[jj]);
-          d32 = __fsqrt_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)));
-          rel = 2e-6f;
-          abs_part = 1e-6f;
-          magk = 9.536743e-7f * S;  // 2^-20 S
-        }
-        // One entry of type t: rounded in float32 when sure, else queued for float64.
-        auto emit = [&](int t, float kt, int32_t* rowt) {
-          int32_t v;
-          const bool sure = round_screened(__fmul_rn(d32, kt), rel, kt * magk + abs_part, v) && screen;
-          if (live && sure) rowt[j] = v;
-          const unsigned need = __ballot_sync(0xffffffffu, live && !sure);
-          if (need) {
-            if (n + 32 > kQueue) {
-              drain(P, c, base, L, LL, q, n, lane, bad);
-              n = 0;
-            }
-            if (live && !sure) q[n + __popc(need & ((1u << lane) - 1u))] = (i << 12) | (j << 1) | t;
-            n += __popc(need);
+          const float dx = __fadd_rn(__fsub_rn(a.x, bb.x), __fsub_rn(a.z, bb.z));
+          float dy = __fsub_rn(a.y, bb.y), dl = __fsub_rn(a.w, bb.w);
+          // Longitudes more than half a turn apart (either side of the date line): the short way
+          // round, with the difference's own rounding error (Knuth's two-sum) kept, since what is
+          // left may be small.
+          if (fabsf(dy) > 3.14159274f) {
+            const float v = __fsub_rn(dy, a.y);
+            const float err = __fsub_rn(__fsub_rn(a.y, __fsub_rn(dy, v)), __fadd_rn(bb.y, v));
+            const float turn = copysignf(6.28318548f, dy);
+            dl = __fadd_rn(dl, __fadd_rn(err, copysignf(1.74845553e-07f, dy)));  // float(2 pi) is above 2 pi by this
+            dy = __fsub_rn(dy, turn);
           }
-        };
-        emit(0, k0, row);
-        if (nt > 1) emit(1, k1, row1);
+          dy = __fadd_rn(dy, dl);
+          const float s1 = sin_half(__fmul_rn(dx, 0.5f)), s2 = sin_half(__fmul_rn(dy, 0.5f));
+          const float g = __fmaf_rn(__fmul_rn(cphi[il], cj), __fmul_rn(s2, s2), __fmul_rn(s1, s1));
+          const float r = g > 0.0f ? __fmul_rn(g, rsqrtf(g)) : g;  // sqrt(0) = 0 exactly; NaN stays NaN
+          float angle = asin_root(r, g);
+          screen = r <= 0.9f && fmaxf(fabsf(dx), fabsf(dy)) <= 3.1417f;  // else the fits do not hold
+          if (g > 0.25f) angle = asinf(r);
+          d32 = __fmul_rn(two_r32, angle);
+        } else {
+          const float dx = __fsub_rn(a.x, bb.x), dy = __fsub_rn(a.y, bb.y);
+          const float g = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+          d32 = g > 0.0f ? __fmul_rn(g, rsqrtf(g)) : g;
+        }
+        int32_t v0, v1 = 0;
+        const bool sure0 = round_screened_bounded(__fmul_rn(d32, k0), rel, c0, v0) && screen;
+        const bool sure1 = NT < 2 || (round_screened_bounded(__fmul_rn(d32, k1), rel, c1, v1) && screen);
+        if (live && !(sure0 && sure1)) {  // rare: float64, later if the queue has room
+#pragma unroll
+          for (int ty = 0; ty < NT; ++ty) {
+            if (ty == 0 ? sure0 : sure1) continue;
+            const Deferred e{b, i0 + il, j, ty};
+            const unsigned pos = atomicAdd(&s_qn, 1u);
+            if (pos < kTileQueue) {
+              queue[pos] = e;
+            } else {
+              const int32_t v = deferred_value(P, e, bad);
+              if (ty == 0) v0 = v;
+              else v1 = v;
+            }
+          }
+        }
+        if (live) {
+          out[0] = v0;
+          if (NT > 1) out[LL] = v1;
+        }
+        if (!diagonal) {
+          mirror[0][jl][il] = v0;
+          if (NT > 1) mirror[NT - 1][jl][il] = v1;
+        }
       }
     }
-    drain(P, c, base, L, LL, q, n, lane, bad);
+    __syncthreads();
+    const unsigned waiting = s_qn;  // nothing queues before the next tile's first barrier
+    if (!diagonal) {
+      const int cols = min(kTile, L - j0);  // the row block is full: I < J
+      for (int jl = warp; jl < cols; jl += kWarps) {
+        int32_t* out = base + static_cast<int64_t>(j0 + jl) * L + i0 + lane;
+#pragma unroll
+        for (int ty = 0; ty < NT; ++ty) {
+          out[ty * LL] = mirror[ty][jl][lane];
+          out[ty * LL + 32] = mirror[ty][jl][lane + 32];
+        }
+      }
+    }
+    if (waiting >= kTileQueue / 2 || t + 1 == t1) {  // uniform over the block
+      __syncthreads();  // the float32 values of the entries are written
+      const int nq = min(static_cast<int>(waiting), kTileQueue);
+      for (int k = tid; k < nq; k += kThreads) {
+        const Deferred e = queue[k];
+        const int32_t v = deferred_value(P, e, bad);
+        const int eL = P.loc_off[e.b + 1] - P.loc_off[e.b];
+        int32_t* o = P.travel + P.travel_off[e.b] + static_cast<int64_t>(e.t) * eL * eL;
+        o[static_cast<int64_t>(e.i) * eL + e.j] = v;
+        o[static_cast<int64_t>(e.j) * eL + e.i] = v;
+      }
+      __syncthreads();
+      if (tid == 0) s_qn = 0u;
+    }
   }
   if (bad && P.status) atomicExch(P.status, ASCHED_E_INVALID);
 }
@@ -508,7 +633,11 @@ extern "C" int asched_travel_matrix(const asched_travel_spec* spec, int32_t* tra
   int64_t n_small = 0;
   for (int b = 0; b < B; ++b) n_small += is_small(spec->h_loc_off[b + 1] - spec->h_loc_off[b], q.nt);
   const bool hav = q.metric == ASCHED_METRIC_HAVERSINE;
-  if (n_small > 0) {
+  // Fewer small instances than the tile kernel has CTAs join its tiles.
+  const bool skip_small = n_small >= static_cast<int64_t>(sms) * 4;
+  int64_t tiles = 0;
+  for (int b = 0; b < B; ++b) tiles += tiles_of(spec->h_loc_off[b + 1] - spec->h_loc_off[b], q.nt, skip_small);
+  if (skip_small) {
     void (*const kernels[2][2])(MParams) = {{travel_small_kernel<false, 1>, travel_small_kernel<false, 2>},
                                             {travel_small_kernel<true, 1>, travel_small_kernel<true, 2>}};
     void (*const kern)(MParams) = kernels[hav][q.nt - 1];
@@ -524,13 +653,12 @@ extern "C" int asched_travel_matrix(const asched_travel_spec* spec, int32_t* tra
     kern<<<grid, kSmallThreads, 0, st>>>(q);
     if (cudaGetLastError() != cudaSuccess) return ASCHED_E_CUDA;
   }
-  if (n_small < B) {
+  if (tiles > 0) {
+    void (*const kernels[2][2])(MParams, bool, int64_t) = {{travel_tiles_kernel<false, 1>, travel_tiles_kernel<false, 2>},
+                                                           {travel_tiles_kernel<true, 1>, travel_tiles_kernel<true, 2>}};
     const int64_t cap = static_cast<int64_t>(sms) * 4;  // 4 CTAs of 256 threads per SM
-    const int grid = static_cast<int>(B - n_small < cap ? B - n_small : cap);
-    if (hav)
-      travel_kernel<true><<<grid, kThreads, 0, st>>>(q);
-    else
-      travel_kernel<false><<<grid, kThreads, 0, st>>>(q);
+    const int grid = static_cast<int>(tiles < cap ? tiles : cap);
+    kernels[hav][q.nt - 1]<<<grid, kThreads, 0, st>>>(q, skip_small, tiles);
     if (cudaGetLastError() != cudaSuccess) return ASCHED_E_CUDA;
   }
   return ASCHED_OK;
