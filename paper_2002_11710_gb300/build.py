@@ -1,6 +1,6 @@
 """Compile the CUDA library in-tree: paper_2002_11710_gb300/_build/libasched.so.
 
-sm_103a only (GB300); eight translation units compiled in parallel and linked into
+sm_103a only (GB300); nine translation units compiled in parallel and linked into
 one shared library, so it builds in a minute or two here and on the GPU host alike.
 """
 from __future__ import annotations
@@ -11,10 +11,10 @@ import sys
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
-SRCS = [os.path.join(PKG, "csrc", n) for n in ("carry.cu", "batch.cu", "serving.cu", "full.cu", "sweep.cu", "matrix.cu",
-                                                "asched.cu", "peaks.cu")]
+SRCS = [os.path.join(PKG, "csrc", n) for n in ("carry.cu", "batch.cu", "serving.cu", "full.cu", "sweep.cu", "sweep_warp.cu",
+                                                "matrix.cu", "asched.cu", "peaks.cu")]
 HDRS = [os.path.join(ROOT, "include", "asched.h")] + [os.path.join(PKG, "csrc", n) for n in (
-    "nvtx_range.h", "kernels.h", "search.cuh", "carry.cuh", "instance.cuh")]
+    "nvtx_range.h", "kernels.h", "sweep.h", "search.cuh", "carry.cuh", "instance.cuh")]
 OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT_DIR, "libasched.so")
 
