@@ -35,9 +35,7 @@
 //     so any launch shape gives the same trajectory.
 //   * The tabu list is a V x M table of iteration stamps in shared memory.
 //   * The batch and serving kernels run the same search per instance, one CTA or one
-//     cluster each, with one more record per mission (a relocation's source-route
-//     delta), relocation items of four missions and the pass over every pair of
-//     missions in its short form, the swaps of route neighbours in a pass of their own.
+//     cluster each.
 
 #pragma once
 
@@ -613,36 +611,35 @@ template <bool PEN, bool DL, bool BIG>
 __device__ __forceinline__ void write_records(const Smem& sm, const Tab<BIG>& tb, const State& S, const Ctx& c,
                                               int t, int nx, int pv, int vw) {
   // Every load comes before the first store: the stores go to the same shared array, so
-  // the compiler could not move a load above one of them.
+  // the compiler could not move a load above one of them. Missions and route ends take the
+  // same path: this is a chain on one warp that the others wait for.
   const int plane = vw_plane(vw);
   const int tyl = plane * c.L, tym = plane * c.Mp;
+  const bool mission = t < c.M, nm = nx < c.M, pm = pv < c.M;
+  const int tm = mission ? t : 0, nxm = nm ? nx : 0, pvm = pm ? pv : 0;
   const int rowA = tb.row(tyl, sm.eloc[pv]);
   const int rowB = tb.row(tyl, sm.sloc[t]);
+  const int rowBn = tb.row(tyl, sm.sloc[nx]);
+  const int ct = sm.cmat[tym + tm], cx = sm.cmat[tym + nxm];
+  int wt = 0, wx = 0, wp = 0;
+  if (DL) {
+    wt = sm.wm[tm];
+    wx = sm.wm[nxm];
+    wp = sm.wm[pvm];
+  }
+  const int aT = tb.a(rowA, tm), bT = tb.b(rowBn, tm);
+  const int aN = tb.a(rowA, nxm), bP = tb.b(mission ? rowBn : rowB, pvm);
   const int nv = nx | (vw << 13);
-  const int dep = (DL && pv < c.M) ? sm.wm[pv] : 0;
-  if (t < c.M) {
-    const int rowBn = tb.row(tyl, sm.sloc[nx]);
-    const int aT = tb.a(rowA, t);
-    const int bT = tb.b(rowBn, t);
-    const int slot = aT + bT;
-    const int ct = sm.cmat[tym + t];
-    const int cn = nx < c.M ? sm.cmat[tym + nx] : 0;
-    const int leg = nx < c.M ? tb.a(rowA, nx) - cn : (pv < c.M ? tb.b(rowBn, pv) : 0);
-    const int wt = DL ? sm.wm[t] : 0;
-    const int wn = DL ? (nx < c.M ? sm.wm[nx] : c.horizon) : 0;
-    const int rem = leg - slot;
-    S.prv()[t] = pv;
-    S.r2()[t] = make_int2(nv, rem);
-    S.y4()[t] = make_int4(rowA, rowB, aT - ct, nv);
-    S.s4()[t] = make_int4(nv, rowA, rowBn, slot);
-    if (DL) S.d4()[t] = make_int4(dep, wt - ct, wn - cn, (dep + leg + cn <= wn) ? 1 : 0);
-  } else {
-    const int inleg = (pv == t) ? 0 : tb.b(rowB, pv);
-    S.prv()[t] = pv;
-    S.r2()[t] = make_int2(nv, 0);
-    S.y4()[t] = make_int4(rowA, rowB, inleg, nv);
-    S.s4()[t] = make_int4(nv, 0, 0, 0);
-    if (DL) S.d4()[t] = make_int4(dep, c.horizon, 0, 1);
+  const int home = pm ? bP : 0;  // from the previous mission to the end
+  const int leg = nm ? aN - cx : home;
+  const int slot = aT + bT;
+  S.prv()[t] = pv;
+  S.r2()[t] = make_int2(nv, mission ? leg - slot : 0);
+  S.y4()[t] = make_int4(rowA, rowB, mission ? aT - ct : home, nv);
+  S.s4()[t] = make_int4(nv, rowA, rowBn, slot);  // of missions
+  if (DL) {
+    const int dep = pm ? wp : 0, cn = nm ? cx : 0, wn = nm ? wx : c.horizon;
+    S.d4()[t] = mission ? make_int4(dep, wt - ct, wn - cn, dep + leg + cn <= wn ? 1 : 0) : make_int4(dep, c.horizon, 0, 1);
   }
 }
 
@@ -660,7 +657,7 @@ template <bool PEN, bool DL, bool DEBUG, bool HELI>
 __device__ __forceinline__ void reloc_one(const Smem& sm, const State& S, const Ctx& c, int y, int m, int nvm,
                                           int rem, const int4& g, int a, int b, int fy, int stamp, int it,
                                           int zrel, const KParams& P, uint64_t& acc) {
-  const bool valid = (y != m) && (y != nv_next(nvm));
+  const bool valid = (y != m) & (y != nv_next(nvm));
   const int vm = nv_veh(nvm), vy = nv_veh(g.w);
   const int ins = a + b - g.z;
   const int d = rem + ins;
@@ -670,23 +667,26 @@ __device__ __forceinline__ void reloc_one(const Smem& sm, const State& S, const 
   int delta;
   bool feas;
   const int fm = S.fb()[vm];
+  int4 dy = make_int4(0, 0, 0, 0);
+  int w = 0, leave = 1;
+  if (DL) {
+    dy = S.d4()[y];
+    w = sm.wm[m];
+    leave = S.d4()[m].w;
+  }
   if (PEN) {
     const int pen = same ? pos0(fy + d) : pos0(fm + rem) - pos0(fm) + pos0(fy + ins);
     delta = d + c.lam * (pen - pos0(fy));
     feas = true;
   } else {
     delta = d;
-    feas = same ? (fy + d <= 0) : ((fm + rem <= 0) && (fy + ins <= 0));
+    feas = same ? (fy + d <= 0) : ((fm + rem <= 0) & (fy + ins <= 0));
   }
-  if (HELI) feas = feas && !((nvm >> 24) & (g.w >> 23) & 1);  // heli-only m onto a plane
-  if (DL) {
-    const int4 dy = S.d4()[y];
-    const int w = sm.wm[m];
-    feas = feas && (dy.x + a <= w) && (w + b <= dy.y) && S.d4()[m].w;
-  }
+  if (HELI) feas = feas & !((nvm >> 24) & (g.w >> 23) & 1);  // heli-only m onto a plane
+  if (DL) feas = feas & (dy.x + a <= w) & (w + b <= dy.y) & (leave != 0);
   const bool tabu = stamp >= it;
   const bool asp = delta < zrel;
-  const bool adm = valid && feas && (!tabu || asp);
+  const bool adm = valid & feas & (!tabu | asp);
   const uint32_t id = (static_cast<uint32_t>(m) << kIdShift) | static_cast<uint32_t>(y);
   if (DEBUG && valid) {
     const int64_t idx = static_cast<int64_t>(m) * (c.N - 2) + y - (y > m) - (y > nv_next(nvm));
@@ -763,21 +763,21 @@ __device__ __forceinline__ void eval_swap(const Smem& sm, const Tab<BIG>& tb, co
     feas = true;
   } else {
     delta = d;
-    feas = same ? (fa + d <= 0) : ((fa + da <= 0) && (fb + db <= 0));
+    feas = same ? (fa + d <= 0) : ((fa + da <= 0) & (fb + db <= 0));
   }
-  if (HELI) feas = feas && !((((nva >> 24) & (nvb >> 23)) | ((nvb >> 24) & (nva >> 23))) & 1);
+  if (HELI) feas = feas & !((((nva >> 24) & (nvb >> 23)) | ((nvb >> 24) & (nva >> 23))) & 1);
   if (DL) {
     const int4 xa = S.d4()[a], xb = S.d4()[b];
     const int wa = sm.wm[a], wb = sm.wm[b];
     const bool l1 = (q.adjB ? wa : xa.x) + q.t1 <= wb;
-    const bool l2 = q.adjA || (wb + q.t2 <= xa.z);
+    const bool l2 = q.adjA | (wb + q.t2 <= xa.z);
     const bool l3 = (q.adjA ? wb : xb.x) + q.t3 <= wa;
-    const bool l4 = q.adjB || (wa + q.t4 <= xb.z);
-    feas = feas && l1 && l2 && l3 && l4;
+    const bool l4 = q.adjB | (wa + q.t4 <= xb.z);
+    feas = feas & l1 & l2 & l3 & l4;
   }
-  const bool tabu = (tb.tabu(vb, a) >= it) || (tb.tabu(va, b) >= it);
+  const bool tabu = (tb.tabu(vb, a) >= it) | (tb.tabu(va, b) >= it);
   const bool asp = delta < zrel;
-  const bool adm = feas && (!tabu || asp);
+  const bool adm = feas & (!tabu | asp);
   const int m1 = a < b ? a : b, m2 = a < b ? b : a;
   const uint32_t id = kSwapBit | (static_cast<uint32_t>(m1) << kIdShift) | static_cast<uint32_t>(m2);
   if (DEBUG) {
@@ -823,6 +823,111 @@ __device__ __forceinline__ uint64_t eval_items(const Smem& sm, const Tab<BIG>& t
     }
   }
   return key;
+}
+
+// Searches of few items per thread: a thread's relocations (m before y) and its sides of swaps
+// are the same in every iteration, so their coordinates stay in registers. Each swap is shared
+// by two neighbouring lanes: a lane takes its own mission's place (m, with y put there) and
+// they add up by shuffles. An iteration of such a search is the chain of a few items, so its
+// length counts, not the work: pairs of relocations and whole swaps, a lane each, took 1,364
+// cycles of the paper fleet's iteration (24 missions), most of the warps idle.
+constexpr int kNarrowItems = 2;  // per thread at most
+struct NarrowItem {
+  int kind;  // 0: none, 1: relocation, 2: swap, 3: relocations of m and m + 1 (the same for a warp)
+  bool live;
+  int m, y;
+  __device__ __forceinline__ uint32_t pack() const {
+    return static_cast<uint32_t>(kind) << 28 | (live ? 1u << 27 : 0u) | static_cast<uint32_t>(m) << 13 | static_cast<uint32_t>(y);
+  }
+  static __device__ __forceinline__ NarrowItem of(uint32_t w) {
+    return NarrowItem{static_cast<int>(w >> 28), (w >> 27 & 1u) != 0, static_cast<int>(w >> 13 & 0xFFFu),
+                      static_cast<int>(w & 0x1FFFu)};
+  }
+};
+
+// Chunks of 32 items: relocations (singly or of two missions), then sides of swaps.
+__host__ __device__ __forceinline__ int64_t narrow_chunks(int64_t M, int64_t V, bool pairs) {
+  return ((M + V) * (pairs ? (M + 1) / 2 : M) + 31) / 32 + (M * (M - 1) + 31) / 32;
+}
+
+__device__ __forceinline__ NarrowItem narrow_item(int M, int N, bool pairs, int chunk) {
+  const int lane = threadIdx.x & 31;
+  const int H = pairs ? (M + 1) / 2 : M;  // items per node
+  const int R = (N * H + 31) / 32, W = (M * (M - 1) + 31) / 32;
+  NarrowItem n = {0, false, 0, 0};
+  if (chunk < R) {
+    const int i = 32 * chunk + lane;
+    n.kind = pairs ? 3 : 1;
+    n.live = i < N * H;
+    n.y = n.live ? i / H : 0;
+    n.m = n.live ? (i - n.y * H) << (pairs ? 1 : 0) : 0;
+  } else if (chunk < R + W) {
+    const int h = 32 * (chunk - R) + lane;
+    n.kind = 2;
+    n.live = h < M * (M - 1);
+    if (n.live) {  // the pairs (a, a + row + 1 mod M), as in the main loop's swap items
+      const int j = h >> 1, row = j / M, a = j - row * M;
+      const int b = a + row + 1 >= M ? a + row + 1 - M : a + row + 1;
+      n.m = h & 1 ? b : a;
+      n.y = h & 1 ? a : b;
+    }
+  }
+  return n;
+}
+
+template <bool PEN, bool DL, bool BIG>
+__device__ __forceinline__ uint64_t eval_narrow(const Smem& sm, const Tab<BIG>& tb, const State& S, const Ctx& c,
+                                                const NarrowItem& n, int it, int zrel, const KParams& P) {
+  const int m = n.m, y = n.y;
+  if (n.kind == 1) {
+    const int2 r = S.r2()[m];
+    const int4 g = S.y4()[y];
+    const int vy = nv_veh(g.w);
+    const int a = tb.a(g.x, m), b = tb.b(g.y, m), stamp = tb.tabu(vy, m), fy = S.fb()[vy];
+    uint64_t key = kNoKey;
+    reloc_one<PEN, DL, false, true>(sm, S, c, y, m, r.x, r.y, g, a, b, fy, stamp, it, zrel, P, key);
+    return n.live ? key : kNoKey;
+  }
+  if (n.kind == 3) {
+    uint64_t key = kNoKey;
+    eval_relocate_pair<PEN, DL, false, BIG, true>(sm, tb, S, c, y, m, it, zrel, P, key);
+    return n.live ? key : kNoKey;
+  }
+  const int4 s = S.s4()[m];
+  const int nvo = S.nv(y);
+  const int vm = nv_veh(s.x), vo = nv_veh(nvo);
+  const bool before = nv_next(s.x) == y, after = nv_next(nvo) == m;  // m flies just before y, just after it
+  const int own = tb.row(vw_plane(nv_vw(s.x)) * c.L, sm.eloc[m]);
+  const int t1 = tb.a(after ? own : s.y, y), t2 = tb.b(s.z, before ? m : y);
+  const int f = S.fb()[vm];
+  const bool tabu = tb.tabu(vo, m) >= it;
+  int4 x = make_int4(0, 0, 0, 0);
+  int wm = 0, wo = 0;
+  if (DL) {
+    x = S.d4()[m];
+    wm = sm.wm[m];
+    wo = sm.wm[y];
+  }
+  const int mine = t1 + t2 - s.w, other = __shfl_xor_sync(0xffffffffu, mine, 1);
+  const int d = mine + other;
+  const bool same = vm == vo;
+  int delta = d;
+  bool ok = !((s.x >> 24) & (nvo >> 23) & 1);  // heli-only m onto a plane
+  if (PEN) {
+    const int p0 = pos0(f);
+    const int pen = pos0(f + mine) - p0;
+    const int both = pen + __shfl_xor_sync(0xffffffffu, pen, 1);
+    delta = d + c.lam * (same ? pos0(f + d) - p0 : both);
+  } else {
+    ok = ok & (f + (same ? d : mine) <= 0);
+  }
+  if (DL) ok = ok & ((after ? wm : x.x) + t1 <= wo) & (before | (wo + t2 <= x.z));
+  const unsigned pair = 3u << (threadIdx.x & 30);
+  const bool feas = !(__ballot_sync(0xffffffffu, !ok) & pair);
+  const bool barred = (__ballot_sync(0xffffffffu, tabu) & pair) != 0;
+  const int m1 = m < y ? m : y, m2 = m < y ? y : m;
+  const uint64_t k = pack_key(delta, kSwapBit | (static_cast<uint32_t>(m1) << kIdShift) | static_cast<uint32_t>(m2));
+  return n.live & feas & (!barred | (delta < zrel)) ? k : kNoKey;
 }
 
 // Flight after move `id` of the source route (src) or of the target route (!src): the
@@ -1533,6 +1638,19 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
       }
     }
     const ItemCursor cursor{r_y, r_h, s_j, s_row, s_a, Gq, Gr, Sq, Sr, G, H, Sn};
+    // One item a thread, with relocations singly if they fit, else two missions an item; or two.
+    // Measured on single searches, narrow against the general lists: 10 missions (6 warps,
+    // pairs) 291 -> 209 us for 200 iterations; 24 missions of the paper's fleet (64 warps, one
+    // round) 1,734 -> 1,079 us for 1,000; 61 missions (192 warps, pairs) 1,754 -> 1,589 us with
+    // the copies. Up to four rounds lost: 100 missions (3.6 rounds) 8.7 ms against 7.7 ms.
+    const int64_t threads32 = static_cast<int64_t>(CT) * nwarps;
+    const int64_t single = narrow_chunks(M, V, false), paired = narrow_chunks(M, V, true);
+    const bool narrow = !DEBUG && (single <= kNarrowItems * threads32);
+    const bool pairs = single > threads32 && paired <= threads32;
+    uint32_t item[kNarrowItems];
+#pragma unroll
+    for (int k = 0; k < kNarrowItems; ++k)
+      item[k] = narrow ? narrow_item(M, N, pairs, cid * C + rank + CT * (warp + nwarps * k)).pack() : 0u;
     const int iters = DEBUG ? 1 : P.iterations;
     bool copy_best = false;  // the last move improved the best schedule
     for (it = 0; it < iters; ++it) {
@@ -1543,8 +1661,21 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
       // delta lies well inside the int32 range, so the clamp changes no comparison)
       const int64_t zr = static_cast<int64_t>(zb_eval) - Z;
       const int zrel = static_cast<int>(zr < INT32_MIN ? INT32_MIN : (zr > INT32_MAX ? INT32_MAX : zr));
-      uint64_t key = c.heli ? eval_items<PEN, DL, DEBUG, BIG, true>(sm, tb, S, c, cursor, it_eval, zrel, P)
-                            : eval_items<PEN, DL, DEBUG, BIG, false>(sm, tb, S, c, cursor, it_eval, zrel, P);
+      uint64_t key = kNoKey;
+      if (narrow) {
+        // one after another through the same code: unrolled, the copies outgrow the instruction cache
+        uint32_t i0 = item[0], i1 = item[1];
+        static_assert(kNarrowItems == 2, "the items above");
+#pragma unroll 1
+        while (i0 != 0u) {
+          key = min_u64(key, eval_narrow<PEN, DL, BIG>(sm, tb, S, c, NarrowItem::of(i0), it, zrel, P));
+          i0 = i1;
+          i1 = 0u;
+        }
+      } else {
+        key = c.heli ? eval_items<PEN, DL, DEBUG, BIG, true>(sm, tb, S, c, cursor, it_eval, zrel, P)
+                     : eval_items<PEN, DL, DEBUG, BIG, false>(sm, tb, S, c, cursor, it_eval, zrel, P);
+      }
       if (copy_best) {
         for (int t = tid; t < N; t += nthr) sm.best[t] = nv_next(S.nv(t));
       }
