@@ -1641,7 +1641,7 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
     // One item a thread, with relocations singly if they fit, else two missions an item; or two.
     // Measured on single searches, narrow against the general lists: 10 missions (6 warps,
     // pairs) 291 -> 209 us for 200 iterations; 24 missions of the paper's fleet (64 warps, one
-    // round) 1,734 -> 1,079 us for 1,000; 61 missions (192 warps, pairs) 1,754 -> 1,589 us with
+    // round) 1,734 -> 1,074 us for 1,000; 61 missions (192 warps, pairs) 1,754 -> 1,589 us with
     // the copies. Up to four rounds lost: 100 missions (3.6 rounds) 8.7 ms against 7.7 ms.
     const int64_t threads32 = static_cast<int64_t>(CT) * nwarps;
     const int64_t single = narrow_chunks(M, V, false), paired = narrow_chunks(M, V, true);
@@ -1694,16 +1694,53 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
       } else {
         // ---- apply the chosen move, in place: a node's records depend only on its own links
         // and vehicle and on static tables, so at most six nodes change. One warp rewrites
-        // them, a node per lane, another takes the routes' new flights and the stamps; the
-        // others go straight to the last barrier.
-        // (Every warp rewriting the changed routes' nodes it owns, between two barriers, ran
-        // the same chain on all of them: 1,214 cycles of an iteration on the paper-shaped
-        // instance.)
+        // them, a node per lane, another takes the routes' new flights, a third (if there is
+        // one) the stamps and the trajectory; the others go straight to the last barrier,
+        // where all wait for the longest of these chains. (Every warp rewriting the changed
+        // routes' nodes it owns, between two barriers, took 1,214 cycles of an iteration on
+        // the paper-shaped instance; with flights and stamps on one warp and the trajectory
+        // on the nodes' 870.)
         const bool moved = !timed_out && !bad_key && gk != kNoKey;
         const uint32_t id = static_cast<uint32_t>(gk);
         const bool is_swap = (id & kSwapBit) != 0;
-        // the move's nodes (relocation: m = n1 before y = n2; swap: a = n1, b = n2)
-        const int n1 = static_cast<int>((id >> kIdShift) & kIdMask), n2 = static_cast<int>(id & kIdMask);
+        // the move's nodes (relocation: m = n1 before y = n2; swap: a = n1, b = n2); node 0
+        // without a move, so that the loads below need not wait for that to be known
+        const int n1 = moved ? static_cast<int>((id >> kIdShift) & kIdMask) : 0, n2 = moved ? static_cast<int>(id & kIdMask) : 0;
+        const int wstamp = nwarps > 2 ? 2 : 1;
+        const int readers = nwarps > 2 ? 96 : 64;  // threads that read the move's records before warp 0 writes
+        if (warp == 0) {
+          const int nv1 = S.nv(n1), nv2 = S.nv(n2);
+          const int p1 = S.prv()[n1], p2 = S.prv()[n2];
+          const int x1 = nv_next(nv1), x2 = nv_next(nv2);
+          int t = n1;
+          if (lane == 1) t = n2;
+          if (lane == 2) t = p1;
+          if (lane == 3) t = x1;
+          if (lane == 4) t = p2;
+          if (lane == 5) t = x2;
+          const int nvt = S.nv(t);
+          int nx = nv_next(nvt), pv = S.prv()[t], vw = nv_vw(nvt);
+          relink(is_swap, n1, n2, p1, x1, p2, x2, nv_vw(nv1), nv_vw(nv2), t, nx, pv, vw);
+          named_sync(1, readers);
+          if (moved && lane < 6) write_records<PEN, DL, BIG>(sm, tb, S, c, t, nx, pv, vw);
+        } else if (warp <= wstamp) {
+          const int va = nv_veh(S.nv(n1)), vb = nv_veh(S.nv(n2));
+          if (warp == 1) {
+            const int f = moved ? moved_flight<BIG>(sm, tb, S, c, id, lane == 0) : 0;
+            named_arrive(1, readers);
+            if (moved && (lane == 0 || (lane == 1 && va != vb))) S.fb()[lane == 0 ? va : vb] = f - c.cap;
+          } else {
+            named_arrive(1, readers);
+          }
+          if (warp == wstamp) {
+            if (moved && (lane == 0 || (lane == 1 && is_swap)))
+              tb.set_tabu(lane == 0 ? va : vb, lane == 0 ? n1 : n2, it + P.tenure);
+            if (lead && lane == 2 && !timed_out) {
+              if (P.traj_move) P.traj_move[it] = gk == kNoKey ? kNullMove : id;
+              if (P.traj_z) P.traj_z[it] = Z + (moved ? key_delta(gk) : 0);
+            }
+          }
+        }
         if (moved) {
           Z += key_delta(gk);
           if (Z < zbest) {
@@ -1712,48 +1749,14 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
             copy_best = true;
           }
         }
-        if (warp == 0) {
-          int t = 0, nx = 0, pv = 0, vw = 0;
-          if (moved) {
-            const int nv1 = S.nv(n1), nv2 = S.nv(n2);
-            const int p1 = S.prv()[n1], p2 = S.prv()[n2];
-            const int x1 = nv_next(nv1), x2 = nv_next(nv2);
-            t = n1;
-            if (lane == 1) t = n2;
-            if (lane == 2) t = p1;
-            if (lane == 3) t = x1;
-            if (lane == 4) t = p2;
-            if (lane == 5) t = x2;
-            const int nvt = S.nv(t);
-            nx = nv_next(nvt);
-            pv = S.prv()[t];
-            vw = nv_vw(nvt);
-            relink(is_swap, n1, n2, p1, x1, p2, x2, nv_vw(nv1), nv_vw(nv2), t, nx, pv, vw);
-          }
-          named_sync(1, 64);  // warp 1 has read the move's records
-          if (moved && lane < 6) write_records<PEN, DL, BIG>(sm, tb, S, c, t, nx, pv, vw);
-        } else if (warp == 1) {
-          int f = 0, va = 0, vb = 0;
-          if (moved) {
-            f = moved_flight<BIG>(sm, tb, S, c, id, lane == 0);
-            va = nv_veh(S.nv(n1));
-            vb = nv_veh(S.nv(n2));
-          }
-          named_arrive(1, 64);
-          if (moved && lane < 2) {
-            if (lane == 0 || va != vb) S.fb()[lane == 0 ? va : vb] = f - c.cap;
-            if (lane == 0) tb.set_tabu(va, n1, it + P.tenure);
-            else if (is_swap) tb.set_tabu(vb, n2, it + P.tenure);
-          }
-        }
-        if (lead && tid == 0 && !timed_out) {
-          if (P.traj_move) P.traj_move[it] = gk == kNoKey ? kNullMove : id;
-          if (P.traj_z) P.traj_z[it] = Z;
-        }
       }
-      if (timed_out || bad_key) sm.misc[MISC_STOP] = bad_key ? ASCHED_E_INVALID : ASCHED_E_TIMEOUT;
-      __syncthreads();
-      if (timed_out || bad_key || (K * C > 1 && sm.misc[MISC_STOP] != 0)) {
+      const bool gone = timed_out || bad_key;  // a warp's own: one may time out alone
+      bool stop = gone;
+      if (K * C > 1) stop = __syncthreads_or(gone);
+      else __syncthreads();
+      if (stop) {
+        if (gone) sm.misc[MISC_STOP] = bad_key ? ASCHED_E_INVALID : ASCHED_E_TIMEOUT;
+        __syncthreads();
         status = sm.misc[MISC_STOP];
         break;
       }
