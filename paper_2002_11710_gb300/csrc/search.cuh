@@ -1706,6 +1706,14 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
         // the move's nodes (relocation: m = n1 before y = n2; swap: a = n1, b = n2); node 0
         // without a move, so that the loads below need not wait for that to be known
         const int n1 = moved ? static_cast<int>((id >> kIdShift) & kIdMask) : 0, n2 = moved ? static_cast<int>(id & kIdMask) : 0;
+        if (moved) {
+          Z += key_delta(gk);
+          if (Z < zbest) {
+            zbest = Z;
+            best_it = it;
+            copy_best = true;
+          }
+        }
         const int wstamp = nwarps > 2 ? 2 : 1;
         const int readers = nwarps > 2 ? 96 : 64;  // threads that read the move's records before warp 0 writes
         if (warp == 0) {
@@ -1737,16 +1745,8 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
               tb.set_tabu(lane == 0 ? va : vb, lane == 0 ? n1 : n2, it + P.tenure);
             if (lead && lane == 2 && !timed_out) {
               if (P.traj_move) P.traj_move[it] = gk == kNoKey ? kNullMove : id;
-              if (P.traj_z) P.traj_z[it] = Z + (moved ? key_delta(gk) : 0);
+              if (P.traj_z) P.traj_z[it] = Z;
             }
-          }
-        }
-        if (moved) {
-          Z += key_delta(gk);
-          if (Z < zbest) {
-            zbest = Z;
-            best_it = it;
-            copy_best = true;
           }
         }
       }
