@@ -217,71 +217,89 @@ __device__ __forceinline__ Mine load_mine(const CarryCtx& c, int m, int v) {
   return r;
 }
 
+constexpr int64_t kNoSwap = INT64_MAX;
+// What the lane's mission reads for node y, all of it for every node (of a route's end too),
+// so that two nodes' loads can go side by side: with 8 or 16 warps an SM a node is a chain of
+// dependent loads. One node at a time, with branches: 1,024 mixed instances 57.8 ms, one of 193
+// missions on 3 vehicles alone 46.2 ms; without branches 56.7 and 40.3; two at a time 52.3 and
+// 38.1 (with a branch around an odd last one, or a loop of its own for short slices, 56 ms:
+// the larger body, and the two evaluations no longer interleaved).
+struct NodeTimes {
+  int4 x, q, dy;
+  int a, b, b2, a3, b3, own, wy;
+  uint32_t set;
+};
+template <bool DL, class TT>
+__device__ __forceinline__ NodeTimes load_node(const CarryCtx& c, const Mine& r, int y) {
+  NodeTimes t;
+  t.x = ld4(c.rec + 8 * y);
+  t.q = ld4(c.rec + 8 * y + 4);
+  if (DL) {
+    t.dy = ld4(c.d4 + 4 * y);
+    t.wy = g_smem[c.wm + y];
+  }
+  t.own = g_smem[r.ownM + y];
+  t.set = static_cast<uint32_t>(g_smem[c.tb + (c.VW == 1 ? 0 : (r.vm >> 5) * c.Mp) + y]);
+  t.a = tmat<TT>(t.x.y + r.sB) + r.cm;
+  t.b = tmat<TT>(r.rD + t.q.z);
+  t.b2 = tmat<TT>(r.rD + t.x.z);
+  t.a3 = tmat<TT>(r.rowE + t.q.z) + t.own;
+  t.b3 = tmat<TT>(r.layM + t.q.w + r.snB);
+  return t;
+}
 // The lane's mission against node y of the vehicle: the detour key of m before y is taken
 // into ki, (delta, y) of the swap of m and y into wk, or into wt when y is tabu on v(m) (for a
 // given m, swap ids order as y).
-constexpr int64_t kNoSwap = INT64_MAX;
 template <bool PEN, bool DL, class TT>
-__device__ __forceinline__ void eval_node(const CarryCtx& c, const Mine& r, int y, uint32_t& ki, int64_t& wk,
-                                          int64_t& wt) {
-  const int4 x = ld4(c.rec + 8 * y), q = ld4(c.rec + 8 * y + 4);
-  int4 dy;
-  if (DL) dy = ld4(c.d4 + 4 * y);
-  const int a = tmat<TT>(x.y + r.sB) + r.cm;
-  const int b = tmat<TT>(r.rD + q.z);
+__device__ __forceinline__ void eval_node(const CarryCtx& c, const Mine& r, int y, const NodeTimes& n, uint32_t& ki,
+                                          int64_t& wk, int64_t& wt) {
+  const int a = n.a, b = n.b;
   const bool mfirst = y == r.next, self = y == r.m;
   {
-    const uint32_t k = static_cast<uint32_t>(a + b - q.x + static_cast<int>(c.add)) * c.mul + static_cast<uint32_t>(y);
-    bool ok = !mfirst && !self;
-    if (DL) ok = ok && dy.x + a <= r.w && r.w + b <= dy.y;
-    if (ok && k < ki) ki = k;
+    const uint32_t k = static_cast<uint32_t>(a + b - n.q.x + static_cast<int>(c.add)) * c.mul + static_cast<uint32_t>(y);
+    bool ok = !mfirst & !self;
+    if (DL) ok = ok & (n.dy.x + a <= r.w) & (r.w + b <= n.dy.y);
+    ki = ok & (k < ki) ? k : ki;
   }
-  if (y < c.M) {
-    const uint32_t set = static_cast<uint32_t>(g_smem[c.tb + (c.VW == 1 ? 0 : (r.vm >> 5) * c.Mp) + y]);
-    const int b2 = tmat<TT>(r.rD + x.z);
-    const int a3 = tmat<TT>(r.rowE + q.z) + g_smem[r.ownM + y];
-    const int b3 = tmat<TT>(r.layM + q.w + r.snB);
-    int da = a + b2 - x.w, db = a3 + b3 - r.slot;
-    // Neighbours fly straight from one to the other, in the other direction than before: with
-    // f before s, the new cost is (prev f -> s) + (s -> f) + (f -> next s) against both slots,
-    // which count the old leg (f -> s) twice.
-    const bool yfirst = nv_next(x.x) == r.m;
-    int am = a, ay = a3;  // flights into m and y in their new places
-    if (mfirst | yfirst) {
-      const int back = tmat<TT>(r.layM + q.w + r.sB);  // from y's delivery to m's pickup
-      if (mfirst) {
-        am = back + r.cm;
-        da = am + b2 - x.w;
-        db = a3 + b - r.slot;
-      } else {
-        ay = b + g_smem[r.ownM + y];
-        da = a + back - x.w;
-        db = ay + b3 - r.slot;
-      }
-    }
-    const int d = da + db;
-    int delta;
-    bool ok = !self && !(x.x & r.hmask);
-    if (PEN) {
-      const int gv = r.same ? d : da, gm = r.same ? 0 : db;
-      delta = d + c.lam * (pos0(r.fv + gv) + pos0(r.fm + gm) - r.p0);
+  int da = a + n.b2 - n.x.w, db = n.a3 + n.b3 - r.slot;
+  // Neighbours fly straight from one to the other, in the other direction than before: with
+  // f before s, the new cost is (prev f -> s) + (s -> f) + (f -> next s) against both slots,
+  // which count the old leg (f -> s) twice.
+  const bool yfirst = nv_next(n.x.x) == r.m;
+  int am = a, ay = n.a3;  // flights into m and y in their new places
+  if ((mfirst | yfirst) & (y < c.M)) {
+    const int back = tmat<TT>(r.layM + n.q.w + r.sB);  // from y's delivery to m's pickup
+    if (mfirst) {
+      am = back + r.cm;
+      da = am + n.b2 - n.x.w;
+      db = n.a3 + b - r.slot;
     } else {
-      delta = d;
-      ok = ok && (r.same ? r.fv + d <= 0 : (r.fv + da <= 0 && r.fm + db <= 0));
+      ay = b + n.own;
+      da = a + back - n.x.w;
+      db = ay + n.b3 - r.slot;
     }
-    if (DL) {
-      const int wy = g_smem[c.wm + y];
-      const bool l1 = (mfirst ? wy : dy.x) + am <= r.w;
-      const bool l2 = yfirst || r.w + b2 <= dy.z;
-      const bool l3 = (yfirst ? r.w : r.d.x) + ay <= wy;
-      const bool l4 = mfirst || wy + b3 <= r.d.z;
-      ok = ok && l1 && l2 && l3 && l4;
-    }
-    const int64_t k = (static_cast<int64_t>(delta) << 32) | y;
-    const bool barred = (set & r.vbit) != 0;
-    if (ok && !barred && k < wk) wk = k;
-    if (ok && barred && k < wt) wt = k;
   }
+  const int d = da + db;
+  int delta;
+  bool ok = (y < c.M) & !self & !(n.x.x & r.hmask);
+  if (PEN) {
+    const int gv = r.same ? d : da, gm = r.same ? 0 : db;
+    delta = d + c.lam * (pos0(r.fv + gv) + pos0(r.fm + gm) - r.p0);
+  } else {
+    delta = d;
+    ok = ok & (r.same ? r.fv + d <= 0 : ((r.fv + da <= 0) & (r.fm + db <= 0)));
+  }
+  if (DL) {
+    const bool l1 = (mfirst ? n.wy : n.dy.x) + am <= r.w;
+    const bool l2 = yfirst | (r.w + n.b2 <= n.dy.z);
+    const bool l3 = (yfirst ? r.w : r.d.x) + ay <= n.wy;
+    const bool l4 = mfirst | (n.wy + n.b3 <= r.d.z);
+    ok = ok & l1 & l2 & l3 & l4;
+  }
+  const int64_t k = (static_cast<int64_t>(delta) << 32) | y;
+  const bool barred = (n.set & r.vbit) != 0;
+  wk = ok & !barred & (k < wk) ? k : wk;
+  wt = ok & barred & (k < wt) ? k : wt;
 }
 
 // The key of the lane's least swap.
@@ -320,7 +338,7 @@ __device__ __noinline__ uint64_t all_swaps(const CarryCtx c, int x) {
     const Mine r = load_mine<PEN, DL>(c, x, nv_veh(g_smem[c.rec + 8 * y]));
     uint32_t unused = kNoDetour;
     int64_t wk = kNoSwap, wt = kNoSwap;
-    if (!r.barred) eval_node<PEN, DL, TT>(c, r, y, unused, wk, wt);
+    if (!r.barred) eval_node<PEN, DL, TT>(c, r, y, load_node<DL, TT>(c, r, y), unused, wk, wt);
     k = min_u64(k, min_u64(swap_key(x, wk), swap_key(x, wt)));
     least = wt < least ? wt : least;
   }
@@ -469,7 +487,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
       uint32_t ki = kNoDetour;
       int64_t wk = kNoSwap, wt = kNoSwap;
       for (int y = nv_next(S0.nv(M + v));; y = nv_next(S0.nv(y))) {
-        eval_node<PEN, DL, TT>(c, r, y, ki, wk, wt);
+        eval_node<PEN, DL, TT>(c, r, y, load_node<DL, TT>(c, r, y), ki, wk, wt);
         if (y >= M) break;
       }
       if (r.barred) {
@@ -541,9 +559,14 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
               const uint16_t* list = first ? listA : listB;
               const int n = first ? nA : nB;
               const int k0 = (first ? pc : pc - PA) << sh, k1 = k0 + (1 << sh) < n ? k0 + (1 << sh) : n;
-              for (int k = k0 + sub; k < k1; k += subs) eval_node<PEN, DL, TT>(c, r, list[k], ki, wk, wt);
+              for (int k = k0 + sub; k < k1; k += 2 * subs) {  // two nodes' loads side by side (an odd last one twice)
+                const int y0 = list[k], y1 = list[k + subs < k1 ? k + subs : k];
+                const NodeTimes t0 = load_node<DL, TT>(c, r, y0), t1 = load_node<DL, TT>(c, r, y1);
+                eval_node<PEN, DL, TT>(c, r, y0, t0, ki, wk, wt);
+                eval_node<PEN, DL, TT>(c, r, y1, t1, ki, wk, wt);
+              }
             } else if (sub == 0 && r.vm == (e & 0x3FF)) {
-              eval_node<PEN, DL, TT>(c, r, e >> 10, ki, wk, wt);
+              eval_node<PEN, DL, TT>(c, r, e >> 10, load_node<DL, TT>(c, r, e >> 10), ki, wk, wt);
               ki = kNoDetour;
             }
             if (r.barred | !act) {

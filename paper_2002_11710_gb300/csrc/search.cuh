@@ -153,8 +153,8 @@ __host__ __device__ inline Layout make_carry_layout(int M, int V, int L, int nt,
   const int subs = 32 >> y.gm_log;
   y.Sp = y.S | 1;  // odd: 32 vehicles' entries of one mission lie in different banks
   if (y.S <= 32) {
-    // one block of missions: a node per lane group and unit, the entries over all warps
-    y.ulog = 5 - y.gm_log;
+    // one block of missions: two nodes per lane group and unit, the entries over all warps
+    y.ulog = 6 - y.gm_log;
     y.ucap = nwarps;
     y.kv = (V + subs * nwarps - 1) / (subs * nwarps);
     if (y.kv < 4) y.kv = 4;
