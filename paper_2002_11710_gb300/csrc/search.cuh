@@ -24,10 +24,9 @@
 //   * The schedule is a doubly linked list over nodes (missions 0..M-1 and route
 //     ends M..M+V-1), with per-node records (removal delta, gap leg, slot cost,
 //     table row offsets, cap slack, deadline slacks) in an SoA. A node's records
-//     depend only on its own links, vehicle and route flight and on static tables, so
-//     applying a move rewrites them in place, in one pass (one thread per node) after
-//     one barrier that follows the decode: only the nodes of the one or two routes
-//     the move changes are recomputed; the rest are current.
+//     depend only on its own links and vehicle and on static tables, so applying a move
+//     rewrites the at most six relinked nodes in place (one warp, a lane per node), while
+//     another warp takes the two routes' new flights.
 //   * Every move (relocate (m, y) and swap (a, b)) is evaluated in O(1) from the
 //     records and the tables; the per-thread, warp (redux.sync), CTA (shared
 //     memory), cluster (DSMEM) and grid (L2) minimum of the key
