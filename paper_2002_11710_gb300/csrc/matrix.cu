@@ -25,16 +25,18 @@
 //              at 2e-6 t + (60 / speed) 2^-20 S + 1e-6, S the instance's largest |x| + |y|;
 //   Haversine  angles staged as float pairs hi + lo (lo = float(v - hi)), so a difference
 //              (hi_i - hi_j) + (lo_i - lo_j) is within 2 * 2^-24 of itself plus 2^-47 of
-//              the magnitudes. Small instances: half-angle differences, sinf (2 ulp),
-//              squares, cos(phi) staged from float64, sum, square root and asinf (2 ulp)
-//              with its condition number below 1.9 for sqrt(a) <= 0.9 (larger values go to
-//              float64 outright) add below 1.8e-6 relative; screened at
-//              8e-6 t + (60 / speed) 2 r 2^-40 (sum of |angles|) + 1e-5. Tiles: longitudes
-//              more than half a turn apart first take the short way round, so that the
-//              sine's condition number stays below 1; own fits of sine (4 * 2^-24) and
-//              arcsine (asinf where sqrt(a) > 1/2) and cos(phi) within 6 * 2^-24 give
-//              27 * 2^-24 for a and below 2.5e-6 for the time (largest found against
-//              80-bit floats over 14 million pairs, poles and date line among them:
+//              the magnitudes. Longitudes more than half a turn apart first take the short
+//              way round, and latitudes or longitudes still further apart go to float64, so
+//              that the half angle's sine has a condition number below 1 (near a whole turn
+//              it has no bound: without this, the small kernel rounded times between the two
+//              sides of the date line wrongly at 10 km/h; with it 16,384 Haversine instances
+//              of 52 locations take 215 us, 213 before). Small instances: half-angle differences, sinf (2 ulp), squares, cos(phi) staged from float64, sum, square
+//              root and asinf (2 ulp) with its condition number below 1.9 for sqrt(a) <= 0.9
+//              (larger values go to float64 outright) add below 1.8e-6 relative; screened at
+//              8e-6 t + (60 / speed) 2 r 2^-40 (sum of |angles|) + 1e-5. Tiles: own fits of
+//              sine (4 * 2^-24) and arcsine (asinf where sqrt(a) > 1/2) and cos(phi) within
+//              6 * 2^-24 give 27 * 2^-24 for a and below 2.5e-6 for the time (largest found
+//              against 80-bit floats over 14 million pairs, poles and date line among them:
 //              8.8e-7, 0.22 of the screen); screened at 4e-6 t + the same rest.
 // Times of 2^22 minutes or more also go to float64 (small instances: every entry of an
 // instance whose largest possible time, 2 S * 60 / speed or pi r * 60 / speed, is not
@@ -155,6 +157,24 @@ __device__ __forceinline__ bool round_screened_bounded(float t32, float rel, flo
   const float gap = __fsub_rn(0.5f, fabsf(__fsub_rn(t32, __fsub_rn(s, 12582912.0f))));
   v = __float_as_int(s) - 0x4B400000;
   return gap > __fmaf_rn(rel, t32, c);
+}
+
+// Difference of two staged longitudes in radians, (x hi, y hi, x lo, y lo) each. Longitudes
+// more than half a turn apart (either side of the date line) take the short way round, with
+// the difference's own rounding error (Knuth's two-sum) kept, since what is left may be small.
+// The half angle's sine has a condition number below 1 only up to half a turn: what is still
+// beyond it (angles outside a turn) goes to float64.
+constexpr float kHalfTurn = 3.1417f;  // pi (1 + 2^-15)
+__device__ __forceinline__ float longitude_gap(const float4& a, const float4& b) {
+  float d = __fsub_rn(a.y, b.y), low = __fsub_rn(a.w, b.w);
+  if (fabsf(d) > 3.14159274f) {
+    const float v = __fsub_rn(d, a.y);
+    const float err = __fsub_rn(__fsub_rn(a.y, __fsub_rn(d, v)), __fadd_rn(b.y, v));
+    const float turn = copysignf(6.28318548f, d);
+    low = __fadd_rn(low, __fadd_rn(err, copysignf(1.74845553e-07f, d)));  // float(2 pi) is above 2 pi by this
+    d = __fsub_rn(d, turn);
+  }
+  return __fadd_rn(d, low);
 }
 
 // One deferred entry of a small instance: the pair (i, j), i <= j, of type t goes to both
@@ -282,11 +302,11 @@ __global__ void __launch_bounds__(kSmallThreads, 8) travel_small_kernel(const __
       bool screen = true;
       if (HAV) {
         const float dx = __fadd_rn(__fsub_rn(a.x, bb.x), __fsub_rn(a.z, bb.z));
-        const float dy = __fadd_rn(__fsub_rn(a.y, bb.y), __fsub_rn(a.w, bb.w));
+        const float dy = longitude_gap(a, bb);
         const float s1 = sinf(__fmul_rn(dx, 0.5f)), s2 = sinf(__fmul_rn(dy, 0.5f));
         const float h = __fadd_rn(__fmul_rn(s1, s1), __fmul_rn(__fmul_rn(st.cphi[i], st.cphi[j]), __fmul_rn(s2, s2)));
         const float r = __fsqrt_rn(h);
-        screen = r <= 0.9f;
+        screen = r <= 0.9f && fmaxf(fabsf(dx), fabsf(dy)) <= kHalfTurn;
         d32 = __fmul_rn(two_r32, asinf(r));
         const float magk = two_r32 * 9.094947e-13f *  // 2 r 2^-40 (sum of |angles|)
                            (fabsf(a.x) + fabsf(bb.x) + fabsf(a.y) + fabsf(bb.y));
@@ -499,23 +519,12 @@ __global__ void __launch_bounds__(kThreads, 4) travel_tiles_kernel(const __grid_
         bool screen = true;
         if (HAV) {
           const float dx = __fadd_rn(__fsub_rn(a.x, bb.x), __fsub_rn(a.z, bb.z));
-          float dy = __fsub_rn(a.y, bb.y), dl = __fsub_rn(a.w, bb.w);
-          // Longitudes more than half a turn apart (either side of the date line): the short way
-          // round, with the difference's own rounding error (Knuth's two-sum) kept, since what is
-          // left may be small.
-          if (fabsf(dy) > 3.14159274f) {
-            const float v = __fsub_rn(dy, a.y);
-            const float err = __fsub_rn(__fsub_rn(a.y, __fsub_rn(dy, v)), __fadd_rn(bb.y, v));
-            const float turn = copysignf(6.28318548f, dy);
-            dl = __fadd_rn(dl, __fadd_rn(err, copysignf(1.74845553e-07f, dy)));  // float(2 pi) is above 2 pi by this
-            dy = __fsub_rn(dy, turn);
-          }
-          dy = __fadd_rn(dy, dl);
+          const float dy = longitude_gap(a, bb);
           const float s1 = sin_half(__fmul_rn(dx, 0.5f)), s2 = sin_half(__fmul_rn(dy, 0.5f));
           const float g = __fmaf_rn(__fmul_rn(cphi[il], cj), __fmul_rn(s2, s2), __fmul_rn(s1, s1));
           const float r = g > 0.0f ? __fmul_rn(g, rsqrtf(g)) : g;  // sqrt(0) = 0 exactly; NaN stays NaN
           float angle = asin_root(r, g);
-          screen = r <= 0.9f && fmaxf(fabsf(dx), fabsf(dy)) <= 3.1417f;  // else the fits do not hold
+          screen = r <= 0.9f && fmaxf(fabsf(dx), fabsf(dy)) <= kHalfTurn;  // else the fits do not hold
           if (g > 0.25f) angle = asinf(r);
           d32 = __fmul_rn(two_r32, angle);
         } else {
