@@ -30,7 +30,8 @@
 //              that the half angle's sine has a condition number below 1 (near a whole turn
 //              it has no bound: without this, the small kernel rounded times between the two
 //              sides of the date line wrongly at 10 km/h; with it 16,384 Haversine instances
-//              of 52 locations take 215 us, 213 before). Small instances: half-angle differences, sinf (2 ulp), squares, cos(phi) staged from float64, sum, square
+//              of 52 locations take 215 us, 213 before). Small instances: half-angle
+//              differences, sinf (2 ulp), squares, cos(phi) staged from float64, sum, square
 //              root and asinf (2 ulp) with its condition number below 1.9 for sqrt(a) <= 0.9
 //              (larger values go to float64 outright) add below 1.8e-6 relative; screened at
 //              8e-6 t + (60 / speed) 2 r 2^-40 (sum of |angles|) + 1e-5. Tiles: own fits of
@@ -55,8 +56,8 @@
 // exactly, products commute), so each unordered pair is evaluated once and written to
 // (i, j) and (j, i). Two kernels share a batch:
 //   Small instances (n_types * L^2 + 3 <= kOut words, L <= kSmallLoc: L <= 55 for two
-//   types, 78 for one), where a batch has enough of them to fill the chip (4 per SM; fewer
-//   join the tiles), are built whole in shared memory by 128-thread CTAs, eight per SM, one
+//   types, 78 for one), where a batch holds no others or enough of them to fill the chip (a
+//   few among larger ones join the tiles), are built whole in shared memory by 128-thread CTAs, eight per SM, one
 //   CTA per instance (grid-stride), with its coordinates staged once.
 //   The L (L + 1) / 2 pairs are numbered row by row with row
 //   i folded onto row L - 1 - i (L + 1 pairs per folded row), so the threads take
@@ -642,10 +643,24 @@ extern "C" int asched_travel_matrix(const asched_travel_spec* spec, int32_t* tra
   int64_t n_small = 0;
   for (int b = 0; b < B; ++b) n_small += is_small(spec->h_loc_off[b + 1] - spec->h_loc_off[b], q.nt);
   const bool hav = q.metric == ASCHED_METRIC_HAVERSINE;
-  // Fewer small instances than the tile kernel has CTAs join its tiles.
-  const bool skip_small = n_small >= static_cast<int64_t>(sms) * 4;
+  // Small instances take their own kernel where they are all the batch holds or fill the chip
+  // (4 per SM); a few among larger ones join the tiles, which saves a launch and its tail. Per
+  // call, own kernel against tiles: 300 instances of 20 locations 8.4 against 10.4 us, of 52 with
+  // two types 10.5 against 12.5, of 78 12.5 against 16.6 (Haversine 20.8 against 27.9). An
+  // instance wider than a tile is three tiles, so where there is no more than one per SM the
+  // tiles spread it better: 64 of 78 locations 12.5 against 12.0, Haversine 19.5 against 17.7.
+  bool skip_small = n_small >= static_cast<int64_t>(sms) * 4;
+  if (!skip_small && n_small == B) {
+    int widest = 0;
+    for (int b = 0; b < B; ++b) {
+      const int L = spec->h_loc_off[b + 1] - spec->h_loc_off[b];
+      widest = L > widest ? L : widest;
+    }
+    skip_small = widest <= kTile || n_small > sms;
+  }
   int64_t tiles = 0;
-  for (int b = 0; b < B; ++b) tiles += tiles_of(spec->h_loc_off[b + 1] - spec->h_loc_off[b], q.nt, skip_small);
+  if (!skip_small || n_small < B)
+    for (int b = 0; b < B; ++b) tiles += tiles_of(spec->h_loc_off[b + 1] - spec->h_loc_off[b], q.nt, skip_small);
   if (skip_small) {
     void (*const kernels[2][2])(MParams) = {{travel_small_kernel<false, 1>, travel_small_kernel<false, 2>},
                                             {travel_small_kernel<true, 1>, travel_small_kernel<true, 2>}};

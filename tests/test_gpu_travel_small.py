@@ -38,6 +38,16 @@ def test_small_instances_across_the_date_line(region, speeds):
 def test_both_builds_agree(region):
     coords = _coords(region, 640, 30, 55)
     many = _build(coords, [10.0], api.METRIC_HAVERSINE)
-    for k in range(0, 640, 64):  # 64 instances join the tiles
-        for a, b in zip(_build(coords[k:k + 64], [10.0], api.METRIC_HAVERSINE), many[k:k + 64]):
+    large = _coords(region, 1, 90, 90)
+    for k in range(0, 640, 64):  # 64 instances beside a larger one join its tiles
+        for a, b in zip(_build(coords[k:k + 64] + large, [10.0], api.METRIC_HAVERSINE), many[k:k + 64]):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("lo,hi,n", [(1, 20, 9), (30, 64, 64), (65, 78, 64), (65, 78, 200)])
+def test_few_small_instances_alone(lo, hi, n):
+    """Batches of small instances only, too few to fill the chip: by their own kernel up to a
+    tile's side or above one per SM, else by tiles."""
+    _check(_coords("dateline", n, lo, hi), [300.0], "dateline")
+    rng = np.random.default_rng(5)
+    _check([_points(rng, int(rng.integers(lo, hi + 1)), "plane") for _ in range(n)], [300.0], "plane")
