@@ -104,10 +104,11 @@ bool wide_search(const asched_instance* inst) {
   return (evals + 31) / 32 > 4 * 16 * static_cast<int64_t>(kMaxCluster);
 }
 
-// Launch shape: block size, cluster size C and clusters K; returns status.
+// Launch shape (block size, cluster size C and clusters K) and the form of the search it runs
+// (its kernel and layout); returns status.
 // allow_grid: the call has a workspace for the keys between clusters (K may exceed 1).
 int make_plan(const asched_instance* inst, const asched_params* p, bool debug, bool allow_grid,
-              asched_plan_t* plan, Layout* lay_out) {
+              asched_plan_t* plan, Layout* lay_out, void** fn_out) {
   int rc = check_sizes(inst, p);
   if (rc != ASCHED_OK) return rc;
   if (p->grid_clusters < 0 || (!allow_grid && p->grid_clusters > 1)) return ASCHED_E_INVALID;
@@ -185,13 +186,30 @@ int make_plan(const asched_instance* inst, const asched_params* p, bool debug, b
     if (rc != ASCHED_OK) return rc;
     if (K > n) return ASCHED_E_TOO_LARGE;
   }
+  Layout form;
+  const int kind = debug ? SEARCH_TABLES
+                         : pick_search(M, V, inst->n_loc, inst->n_types, inst->deadline != nullptr, cl * K, threads / 32,
+                                       p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0, lay.big, (limit - 64) / 4, &form);
+  if (kind == SEARCH_CARRY32 || kind == SEARCH_CARRY16) {
+    void* cfn = asched_kernels::carry(p->cap_mode == ASCHED_PENALTY, inst->deadline != nullptr, kind == SEARCH_CARRY16);
+    int n = 1;
+    if (cl * K > 1) {
+      rc = active_clusters(cfn, cl, threads, form.total * 4, &n);
+      if (rc != ASCHED_OK) return rc;
+    }
+    if (n >= K) {  // else the full evaluation, which is placed above
+      fn = cfn;
+      lay = form;
+    }
+  }
   plan->cluster_size = cl;
   plan->block_threads = threads;
-  plan->smem_bytes = bytes;
+  plan->smem_bytes = lay.total * 4;
   plan->moves_per_iteration = moves_of(M, V);
   plan->grid_clusters = K;
   plan->workspace_bytes = static_cast<int64_t>(grid_workspace_bytes(K));
   if (lay_out) *lay_out = lay;
+  if (fn_out) *fn_out = fn;
   return ASCHED_OK;
 }
 
@@ -199,7 +217,8 @@ int launch(const asched_instance* inst, const asched_params* p, bool debug, KPar
            size_t ws_bytes, bool allow_grid, void* stream) {
   asched_plan_t plan;
   Layout lay;
-  int rc = make_plan(inst, p, debug, allow_grid, &plan, &lay);
+  void* fn;
+  int rc = make_plan(inst, p, debug, allow_grid, &plan, &lay, &fn);
   if (rc != ASCHED_OK) return rc;
   if (!inst->travel || !inst->veh_base) return ASCHED_E_INVALID;
   if (inst->n_missions > 0 && (!inst->pickup || !inst->delivery)) return ASCHED_E_INVALID;
@@ -207,27 +226,6 @@ int launch(const asched_instance* inst, const asched_params* p, bool debug, KPar
   if (K > 1 && (!workspace || ws_bytes < grid_workspace_bytes(K) || (reinterpret_cast<uintptr_t>(workspace) & 127u)))
     return ASCHED_E_INVALID;
   const bool pen = p->cap_mode == ASCHED_PENALTY;
-  const bool dl = inst->deadline != nullptr;
-  void* fn = asched_kernels::full(pen, dl, debug, lay.big);
-  Layout carry;
-  const int kind =
-      debug ? SEARCH_TABLES
-            : pick_search(inst->n_missions, inst->n_vehicles, inst->n_loc, inst->n_types, dl, plan.cluster_size * K,
-                          plan.block_threads / 32, p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0, lay.big,
-                          (max_smem_optin() - 64) / 4, &carry);
-  if (kind == SEARCH_CARRY32 || kind == SEARCH_CARRY16) {
-    void* cfn = asched_kernels::carry(pen, dl, kind == SEARCH_CARRY16);
-    int n = 1;
-    if (plan.cluster_size * K > 1) {
-      rc = active_clusters(cfn, plan.cluster_size, plan.block_threads, carry.total * 4, &n);
-      if (rc != ASCHED_OK) return rc;
-    }
-    if (n >= K) {  // else the full evaluation, which the plan has placed
-      fn = cfn;
-      lay = carry;
-      plan.smem_bytes = carry.total * 4;
-    }
-  }
   kp.travel = inst->travel;
   kp.veh_base = inst->veh_base;
   kp.veh_type = inst->veh_type;
@@ -608,7 +606,7 @@ int asched_check_instance_host(const asched_instance* inst, const asched_params*
 
 int asched_plan(const asched_instance* inst, const asched_params* params, asched_plan_t* out) {
   if (!out) return ASCHED_E_INVALID;
-  return make_plan(inst, params, false, true, out, nullptr);
+  return make_plan(inst, params, false, true, out, nullptr, nullptr);
 }
 
 namespace {
@@ -642,7 +640,7 @@ int asched_validate(const asched_instance* inst, const asched_params* params) {
 int asched_workspace_bytes(const asched_instance* inst, const asched_params* params, size_t* bytes) {
   if (!bytes) return ASCHED_E_INVALID;
   asched_plan_t plan;
-  const int rc = make_plan(inst, params, false, true, &plan, nullptr);
+  const int rc = make_plan(inst, params, false, true, &plan, nullptr, nullptr);
   if (rc != ASCHED_OK) return rc;
   *bytes = static_cast<size_t>(plan.workspace_bytes);
   return ASCHED_OK;
