@@ -186,18 +186,23 @@ int make_plan(const asched_instance* inst, const asched_params* p, bool debug, b
     if (rc != ASCHED_OK) return rc;
     if (K > n) return ASCHED_E_TOO_LARGE;
   }
+  // Carried move values on one cluster only. Over several, an iteration's chain of table
+  // updates comes on top of the exchange through L2, and the full evaluation's share per warp is
+  // small: 7 x 16 CTAs, carried against full, 400 missions and 50 vehicles 8.5 against 6.7 us an
+  // iteration, 800 and 20 16.1 against 11.3, 1,200 and 30 22.9 against 18.5.
   Layout form;
-  const int kind = debug ? SEARCH_TABLES
-                         : pick_search(M, V, inst->n_loc, inst->n_types, inst->deadline != nullptr, cl * K, threads / 32,
-                                       p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0, lay.big, (limit - 64) / 4, &form);
+  const int kind = debug || K > 1 ? SEARCH_TABLES
+                                  : pick_search(M, V, inst->n_loc, inst->n_types, inst->deadline != nullptr, cl,
+                                                threads / 32, p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0,
+                                                lay.big, (limit - 64) / 4, &form);
   if (kind == SEARCH_CARRY32 || kind == SEARCH_CARRY16) {
     void* cfn = asched_kernels::carry(p->cap_mode == ASCHED_PENALTY, inst->deadline != nullptr, kind == SEARCH_CARRY16);
     int n = 1;
-    if (cl * K > 1) {
+    if (cl > 1) {
       rc = active_clusters(cfn, cl, threads, form.total * 4, &n);
       if (rc != ASCHED_OK) return rc;
     }
-    if (n >= K) {  // else the full evaluation, which is placed above
+    if (n > 0) {  // else the full evaluation, which is placed above
       fn = cfn;
       lay = form;
     }

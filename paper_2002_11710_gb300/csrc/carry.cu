@@ -7,14 +7,12 @@ namespace {
 template <bool PEN, bool DL, class TT>
 __global__ void __launch_bounds__(kMaxThreads, 1) carry_kernel(const __grid_constant__ KParams P) {
   const int C = P.cluster;
-  const int K = P.grid_clusters > 1 ? P.grid_clusters : 1;
-  if (!launch_shape_ok(C, K * C)) {  // uniform over the launch: every CTA returns here
+  if (!launch_shape_ok(C, C)) {  // uniform over the launch: every CTA returns here
     if (blockIdx.x == 0 && threadIdx.x == 0 && P.info) P.info[ASCHED_INFO_STATUS] = ASCHED_E_INVALID;
     return;
   }
   const int rank = C > 1 ? static_cast<int>(cluster_rank()) : 0;
-  const int cid = K > 1 ? static_cast<int>(blockIdx.x) / C : 0;
-  carry_solve<PEN, DL, TT>(P, P.lay, C, rank, K, cid);
+  carry_solve<PEN, DL, TT>(P, P.lay, C, rank);
 }
 
 }  // namespace

@@ -350,9 +350,8 @@ __device__ __noinline__ uint64_t all_swaps(const CarryCtx c, int x) {
 // One complete search of the instance in P, as solve_one, with carried move values; lay is a
 // carry layout.
 template <bool PEN, bool DL, class TT>
-__device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay, const int C, const int rank,
-                                            const int K, const int cid) {
-  const bool lead = rank == 0 && cid == 0;
+__device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay, const int C, const int rank) {
+  const bool lead = rank == 0;
   const Smem sm = carve(lay);
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
@@ -387,8 +386,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
   c.Sp = lay.Sp;
   c.VW = lay.VW;
   const int slice = lay.S;  // missions per CTA
-  const int pos = cid * C + rank;
-  c.m0 = pos * slice < M ? pos * slice : M;
+  c.m0 = rank * slice < M ? rank * slice : M;
   c.S = M - c.m0 < slice ? M - c.m0 : slice;
   int status = ASCHED_OK;
 
@@ -538,7 +536,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
         }
         // units: columns, expired stamps, rows, entries of the other missions
         // rows: with one CTA the missions of both lists, else those listed for this CTA's slice
-        const int nE = (ex.x >= 0) + (ex.y >= 0), nRV = (C * K > 1 ? cn.w : nA + nB) * V;
+        const int nE = (ex.x >= 0) + (ex.y >= 0), nRV = (C > 1 ? cn.w : nA + nB) * V;
         const int e1 = (PA + PB) * nblk, e2 = e1 + nE * nblk, e3 = e2 + ((nRV + 31) >> 5), e4 = e3 + PV * nblk;
         for (int u = warp; u < e4; u += nwarps) {
           if (u < e2) {
@@ -596,7 +594,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
             const int x = (u - e2) * 32 + lane;
             const int k = V > 1 ? static_cast<int>(__umulhi(static_cast<uint32_t>(x), vinv)) : x;
             const int v = x - k * V;
-            const int m = x < nRV ? (C * K > 1 ? rows[k] : (k < nA ? listA[k] : listB[k - nA])) : M;
+            const int m = x < nRV ? (C > 1 ? rows[k] : (k < nA ? listA[k] : listB[k - nA])) : M;
             if (m < M && v != va && v != vb) {
               const int i = m - c.m0;
               const int vm = nv_veh(g_smem[c.rec + 8 * m]), rem = g_smem[c.rec + 8 * m + 5];
@@ -675,7 +673,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
       __syncthreads();
       uint64_t gk = warp_min_key(lane < nwarps ? sm.warpkey()[lane] : kNoKey);
       bool timed_out = false;
-      if (C * K > 1) gk = exchange_keys(P, sm, C, rank, K, cid, it, gk, timed_out);
+      if (C > 1) gk = exchange_keys(P, sm, C, rank, 1, 0, it, gk, timed_out);
       const bool bad_key = !timed_out && !key_names_nodes(gk, M, N);
       const bool go = !timed_out && !bad_key;
       const bool moved = go && gk != kNoKey;
@@ -761,7 +759,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
             const int i = t - c.m0;
             if (t < M && i >= 0 && i < c.S) {
               g_smem[c.rb + i] = INT32_MAX;
-              if (C * K > 1) rows[atomicAdd(&g_smem[lay.ccnt + par + 3], 1)] = static_cast<uint16_t>(t);
+              if (C > 1) rows[atomicAdd(&g_smem[lay.ccnt + par + 3], 1)] = static_cast<uint16_t>(t);
             }
           }
         }
@@ -814,7 +812,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
       }
       if (!go) g_smem[stop_word] = bad_key ? ASCHED_E_INVALID : ASCHED_E_TIMEOUT;
       __syncthreads();
-      if (!go || (C * K > 1 && g_smem[stop_word] != 0)) {
+      if (!go || (C > 1 && g_smem[stop_word] != 0)) {
         status = g_smem[stop_word];
         break;
       }

@@ -16,8 +16,8 @@ __device__ __forceinline__ bool search_instance(const KParams& P, int C, int ran
   Layout lay;
   const int kind = pick_search(P.M, P.V, P.L, P.nt, DL, C, blockDim.x >> 5, P.tenure, compact, half, limit_words, &lay);
   if (lay.total > limit_words) return false;
-  if (kind == SEARCH_CARRY32) carry_solve<PEN, DL, CTab32>(P, lay, C, rank, 1, 0);
-  else if (kind == SEARCH_CARRY16) carry_solve<PEN, DL, CTab16>(P, lay, C, rank, 1, 0);
+  if (kind == SEARCH_CARRY32) carry_solve<PEN, DL, CTab32>(P, lay, C, rank);
+  else if (kind == SEARCH_CARRY16) carry_solve<PEN, DL, CTab16>(P, lay, C, rank);
   else if (kind == SEARCH_TABLES) solve_full<PEN, DL, false>(P, lay, C, rank, 1, 0);
   else solve_full<PEN, DL, true>(P, lay, C, rank, 1, 0);
   return true;

@@ -1,6 +1,6 @@
-"""The search with carried move values over several clusters, and its bounded waits, against
-the oracle: slices of every size, empty ones among them, both matrix types, and a key that
-never arrives (needs a GB300)."""
+"""The search with carried move values on one cluster against the oracle: slices of every size,
+empty ones among them, both matrix types, and a key that never arrives; over several clusters
+the full evaluation runs (needs a GB300)."""
 import pytest
 import torch
 
@@ -9,53 +9,58 @@ from test_gpu_parity import _check_solve_vs_oracle
 
 pytestmark = pytest.mark.gpu
 HARD, PENALTY = gen.HARD, gen.PENALTY
-WARPS = 2  # per CTA, at 64 threads
 
 
 def _instance(M, V, **kw):
     return gen.random_instance(131, n_loc=18, n_vehicles=V, n_missions=M, n_types=2, heli_only_frac=0.2, **kw)
 
 
-def _carried(inst, ctas):
-    """More than 6 chunks of 32 items (pairs of relocations, swaps) a warp."""
-    M, V = inst.n_missions, inst.n_vehicles
-    return (M + V) * ((M + 1) // 2) + M * (M - 1) // 2 > 32 * 6 * ctas * WARPS
+def _carried(inst, mode=PENALTY, **kw):
+    """Only the carried form keeps a ring of moves, two words per iteration of tenure."""
+    dp = api.DeviceProblem(inst)
+    smem = [api.plan(dp, api.make_params(t, 50, mode, 1000, block_threads=64, **kw)).smem_bytes for t in (8, 108)]
+    assert smem[1] - smem[0] in (0, 800)
+    return smem[1] > smem[0]
 
 
-# missions, vehicles, CTAs of a cluster, clusters; slices 41, 27, 14, 6 (two CTAs without
-# missions), 4 (two without) and 5 missions
-SHAPES = [(81, 10, 1, 2), (81, 10, 1, 3), (83, 33, 2, 3), (81, 10, 4, 4), (120, 9, 16, 2), (120, 1, 8, 3)]
-
-
-@pytest.mark.parametrize("M,V,cluster,grid", SHAPES)
+# missions, vehicles, CTAs: slices of 75 missions, 75 (the last shorter), 19, 10 and 10 (the last
+# CTA without missions)
+@pytest.mark.parametrize("M,V,cluster", [(150, 30, 2), (149, 33, 2), (151, 40, 8), (151, 60, 16), (150, 60, 16)])
 @pytest.mark.parametrize("compact", [False, True])
-def test_trajectory_over_clusters(M, V, cluster, grid, compact):
+def test_trajectory_on_one_cluster(M, V, cluster, compact):
     inst = _instance(M, V, duty_cap=900, max_minutes=90)
-    if V == 1:  # the one vehicle may be a plane
-        inst = gen.Instance(**{**inst.__dict__, "heli_only": None})
-    assert _carried(inst, cluster * grid)
-    _check_solve_vs_oracle(inst, PENALTY, 8, 90, cluster_size=cluster, grid_clusters=grid, block_threads=32 * WARPS,
-                           compact=compact)
+    kw = dict(cluster_size=cluster, grid_clusters=1, compact=compact)
+    assert _carried(inst, **kw)
+    _check_solve_vs_oracle(inst, PENALTY, 8, 90, block_threads=64, **kw)
 
 
 @pytest.mark.parametrize("mode", [HARD, PENALTY])
-@pytest.mark.parametrize("cluster,grid", [(1, 3), (2, 2), (4, 4)])
-def test_trajectory_over_clusters_with_deadlines(mode, cluster, grid):
-    inst = _instance(81, 34, duty_cap=400, max_minutes=25, deadlines=True, deadline_lo=1000)
-    assert _carried(inst, cluster * grid)
-    _check_solve_vs_oracle(inst, mode, 6, 90, cluster_size=cluster, grid_clusters=grid, block_threads=32 * WARPS)
+@pytest.mark.parametrize("cluster", [1, 2, 8])
+def test_trajectory_on_one_cluster_with_deadlines(mode, cluster):
+    inst = _instance(120, 40, duty_cap=400, max_minutes=20, deadlines=True, deadline_lo=1100)
+    kw = dict(cluster_size=cluster, grid_clusters=1)
+    assert _carried(inst, mode, **kw)
+    _check_solve_vs_oracle(inst, mode, 6, 90, block_threads=64, **kw)
 
 
-@pytest.mark.parametrize("cluster,grid", [(2, 1), (8, 1), (1, 3), (2, 3), (4, 4)])
-def test_withheld_key_times_out(cluster, grid):
-    """A CTA (one cluster) or a cluster (several) that never publishes its first key."""
-    inst = _instance(81, 10, duty_cap=900, max_minutes=90)
-    assert _carried(inst, cluster * grid)
-    params = api.make_params(8, 50, PENALTY, 1000, cluster_size=cluster, grid_clusters=grid, block_threads=32 * WARPS,
-                             timeout_ns=50_000_000)
+@pytest.mark.parametrize("cluster", [2, 8])
+def test_withheld_key_times_out(cluster):
+    """A CTA that never publishes its first key ends every other wait of the carried loop."""
+    inst = _instance(150, 50, duty_cap=900, max_minutes=90)
+    kw = dict(cluster_size=cluster, grid_clusters=1)
+    assert _carried(inst, **kw)
+    params = api.make_params(8, 50, PENALTY, 1000, block_threads=64, timeout_ns=50_000_000, **kw)
     params.flags |= api._lib.TEST_WITHHOLD_KEY
     out = api.solve(api.DeviceProblem(inst), params)
     torch.cuda.synchronize()
     assert int(out.info[api.INFO_STATUS]) == api.E_TIMEOUT
     assert int(out.info[api.INFO_ITERS]) == 0
-    _check_solve_vs_oracle(inst, PENALTY, 8, 50, cluster_size=cluster, grid_clusters=grid, block_threads=32 * WARPS)
+    _check_solve_vs_oracle(inst, PENALTY, 8, 50, block_threads=64, **kw)
+
+
+@pytest.mark.parametrize("cluster,grid", [(1, 2), (4, 4)])
+def test_full_evaluation_over_several_clusters(cluster, grid):
+    inst = _instance(150, 50, duty_cap=900, max_minutes=90)
+    kw = dict(cluster_size=cluster, grid_clusters=grid)
+    assert not _carried(inst, **kw)
+    _check_solve_vs_oracle(inst, PENALTY, 8, 60, block_threads=64, **kw)
