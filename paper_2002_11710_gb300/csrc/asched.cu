@@ -12,16 +12,16 @@ constexpr int kBatchThreads = 256;  // per CTA of a batch, two CTAs per SM
 
 // Shared-memory layout for an instance: the gather tables when they fit, else the
 // int16 matrix (whose stamps limit iterations + tenure to 32,767). What a call accepts
-// follows from it for every search, also those that then carry move values. reserve: words
-// left free beside the layout (batch_reserve for batches and requests).
-int choose_layout(int M, int V, int L, int nt, const asched_params* p, int limit_bytes, int reserve, Layout* out) {
-  const Layout small = make_layout(M, V, L, nt, false);
-  if (!(p->flags & ASCHED_COMPACT_LAYOUT) && static_cast<int64_t>(small.total + reserve) * 4 + 64 <= limit_bytes) {
+// follows from it for every search, also those that then carry move values. rp: the batch and
+// serving kernels' layout, with the RP records.
+int choose_layout(int M, int V, int L, int nt, const asched_params* p, int limit_bytes, bool rp, Layout* out) {
+  const Layout small = make_layout(M, V, L, nt, false, rp);
+  if (!(p->flags & ASCHED_COMPACT_LAYOUT) && static_cast<int64_t>(small.total) * 4 + 64 <= limit_bytes) {
     *out = small;
     return ASCHED_OK;
   }
-  const Layout big = make_layout(M, V, L, nt, true);
-  if (static_cast<int64_t>(big.total + reserve) * 4 + 64 > limit_bytes) return ASCHED_E_TOO_LARGE;
+  const Layout big = make_layout(M, V, L, nt, true, rp);
+  if (static_cast<int64_t>(big.total) * 4 + 64 > limit_bytes) return ASCHED_E_TOO_LARGE;
   if (static_cast<int64_t>(p->iterations) + p->tenure > 32767) return ASCHED_E_TOO_LARGE;
   *out = big;
   return ASCHED_OK;
@@ -116,7 +116,7 @@ int make_plan(const asched_instance* inst, const asched_params* p, bool debug, b
   const int limit = max_smem_optin();
   if (limit < 0) return ASCHED_E_CUDA;
   Layout lay;
-  rc = choose_layout(M, V, inst->n_loc, inst->n_types, p, limit, 0, &lay);
+  rc = choose_layout(M, V, inst->n_loc, inst->n_types, p, limit, false, &lay);
   if (rc != ASCHED_OK) return rc;
   const int bytes = lay.total * 4;
   void* fn = asched_kernels::full(p->cap_mode == ASCHED_PENALTY, inst->deadline != nullptr, debug, lay.big);
@@ -194,7 +194,7 @@ int make_plan(const asched_instance* inst, const asched_params* p, bool debug, b
   const int kind = debug || K > 1 ? SEARCH_TABLES
                                   : pick_search(M, V, inst->n_loc, inst->n_types, inst->deadline != nullptr, cl,
                                                 threads / 32, p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0,
-                                                lay.big, (limit - 64) / 4, &form);
+                                                lay.big, false, (limit - 64) / 4, &form);
   if (kind == SEARCH_CARRY32 || kind == SEARCH_CARRY16) {
     void* cfn = asched_kernels::carry(p->cap_mode == ASCHED_PENALTY, inst->deadline != nullptr, kind == SEARCH_CARRY16);
     int n = 1;
@@ -318,11 +318,10 @@ int launch_batch(const asched_batch* bt, const asched_params* p, const asched_ba
     int rc = check_sizes(&one, p);
     if (rc != ASCHED_OK) return rc;
     Layout lay;
-    rc = choose_layout(one.n_missions, one.n_vehicles, one.n_loc, one.n_types, p, limit,
-                       batch_reserve(one.n_missions, one.n_vehicles), &lay);
+    rc = choose_layout(one.n_missions, one.n_vehicles, one.n_loc, one.n_types, p, limit, true, &lay);
     if (rc != ASCHED_OK) return rc;
     pick_search(one.n_missions, one.n_vehicles, one.n_loc, one.n_types, bt->deadline != nullptr, C, threads / 32,
-                p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0, lay.big, limit_words, &lay);
+                p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0, lay.big, true, limit_words, &lay);
     if (lay.total > max_words) max_words = lay.total;
   }
   const int64_t bytes = static_cast<int64_t>(max_words) * 4;
@@ -444,8 +443,7 @@ int launch_serve(const asched_server* sv, const asched_params* p, int64_t idle_n
   const int limit = max_smem_optin();
   if (limit < 0) return ASCHED_E_CUDA;
   Layout lay;  // the largest request the slots can hold sizes the launch
-  const int reserve = batch_reserve(sv->max_missions, sv->max_vehicles);
-  rc = choose_layout(sv->max_missions, sv->max_vehicles, sv->max_loc, sv->n_types, p, limit, reserve, &lay);
+  rc = choose_layout(sv->max_missions, sv->max_vehicles, sv->max_loc, sv->n_types, p, limit, true, &lay);
   if (rc != ASCHED_OK) return rc;
   // Requests of every size take the layout they ask for (a small request's may be larger than
   // the largest request's), so the launch has all the shared memory a CTA may use.
@@ -481,7 +479,7 @@ int launch_serve(const asched_server* sv, const asched_params* p, int64_t idle_n
   q.slot_words = serve_slot_words(q.Lc, q.Vc, q.Mc, q.nt);
   q.out_words = serve_out_words(q.Vc, q.Mc);
   q.limit_words = limit_words;
-  q.table_words = lay.total + reserve;
+  q.table_words = lay.total;
   q.compact = (p->flags & ASCHED_COMPACT_LAYOUT) ? 1 : 0;
   q.idle_ns = idle_ns;
   q.slot_data = sv->slot_data;

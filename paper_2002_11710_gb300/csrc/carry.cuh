@@ -394,7 +394,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
   if (tid < 16) sm.misc[tid] = 0;
   __syncthreads();
   int any_heli = 0;
-  int bad = load_statics(P, sm, Mp, any_heli);
+  int bad = load_statics(P, sm, Mp, round_up(N + 1, 4), any_heli);
   int maxT = 0;
   if (TT::kBytes == 4) {
     for (int i = tid; i < nt * L * L; i += nthr) {

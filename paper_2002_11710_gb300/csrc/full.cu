@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) tabu_kernel(const __grid_const
   }
   const int rank = C > 1 ? static_cast<int>(cluster_rank()) : 0;
   const int cid = K > 1 ? static_cast<int>(blockIdx.x) / C : 0;
-  solve_one<PEN, DL, DEBUG, BIG>(P, P.lay, C, rank, K, cid);
+  solve_one<PEN, DL, DEBUG, BIG, false>(P, P.lay, C, rank, K, cid);
 }
 
 }  // namespace

@@ -72,12 +72,6 @@ __host__ __device__ inline int serve_out_words(int Vc, int Mc) {
 
 }  // namespace
 
-// Words per node that batches and requests leave free beside the full evaluation's layouts when
-// they decide between the gather tables and the int16 matrix, and what fits at all.
-namespace {
-__host__ __device__ inline int batch_reserve(int M, int V) { return round_up(M + V, 4); }
-}  // namespace
-
 namespace asched_kernels {
 void* full(bool pen, bool dl, bool debug, bool big);  // tabu_kernel: the full evaluation
 void* carry(bool pen, bool dl, bool t16);             // carry_kernel: carried move values

@@ -34,7 +34,9 @@
 //     so any launch shape gives the same trajectory.
 //   * The tabu list is a V x M table of iteration stamps in shared memory.
 //   * The batch and serving kernels run the same search per instance, one CTA or one
-//     cluster each.
+//     cluster each; their item lists take one more record per mission (a relocation's
+//     source-route delta), relocations of four missions at a time and the pass over every
+//     pair of missions in its short form, the swaps of route neighbours in a pass of their own.
 
 #pragma once
 
@@ -66,7 +68,12 @@ constexpr int64_t kDefaultTimeoutNs = 1000000000ll;
 //   Y4[t] = {A row of prev(t), B row of t, leg prev(t) -> t, nv}   relocation, gap side
 //   S4[t] = {nv, A row of prev(t), B row of next(t), slot cost}    swap side
 //   D4[t] = {dep(prev t), arrive-by slack at t, slack at next(t), removal link ok}
-//   PRV[t] previous node; FB[v] flight of vehicle v minus the duty cap.
+//   PRV[t] previous node; FB[v] flight of vehicle v minus the duty cap;
+//   RP[t]  (after FB) a relocation's delta on t's own route when t moves to another
+//          route: removal delta plus lambda times the change of that route's overflow
+//          (penalty mode), or whether the route stays within the cap (hard mode). Kept by
+//          the batch and serving kernels where they evaluate item lists, whose length it
+//          cuts, and not by the single-instance kernel, whose iterations wait on the apply step.
 constexpr int kBufWordsPerNode = 15;
 
 // Two table layouts. Small instances keep location x mission gather tables (int32):
@@ -89,13 +96,13 @@ struct Layout {  // offsets in int32 words from the start of dynamic shared memo
 
 __host__ __device__ inline int round_up(int x, int k) { return (x + k - 1) / k * k; }
 
-__host__ __device__ inline Layout make_layout(int M, int V, int L, int nt, bool big) {
+__host__ __device__ inline Layout make_layout(int M, int V, int L, int nt, bool big, bool rp) {
   Layout y = {};
   y.big = big;
   y.Mp = round_up(M > 0 ? M : 1, 32);
   y.Np = round_up(M + V, 4);
   y.Vp = round_up(V, 4);
-  y.buf = kBufWordsPerNode * y.Np + y.Vp;  // R2 Y4 S4 D4 PRV, FB
+  y.buf = kBufWordsPerNode * y.Np + y.Vp + (rp ? y.Np : 0);  // R2 Y4 S4 D4 PRV, FB, RP
   y.Ls = round_up(L, 2);
   if ((y.Ls / 2) % 2 == 0) y.Ls += 2;
   int o = 0;
@@ -110,7 +117,7 @@ __host__ __device__ inline Layout make_layout(int M, int V, int L, int nt, bool 
   }
   y.cmat = o;    o += nt * y.Mp;
   y.wm = o;      o += y.Mp;
-  y.eloc = o;    o += round_up(M + V + 3, 4);  // pairs of missions read up to M
+  y.eloc = o;    o += round_up(M + V + 3, 4);  // quads of missions read up to M + 2
   y.sloc = o;    o += round_up(M + V + 3, 4);
   y.vtype = o;   o += y.Vp;
   y.tyl = o;     o += y.Vp;
@@ -231,12 +238,16 @@ __host__ __device__ inline Layout make_carry_layout(int M, int V, int L, int nt,
 // The layout of a search: carried move values when they fit (with the int32 matrix, or, where
 // the limits of the int16 matrix hold anyway, the int16 one), else the full evaluation with
 // the gather tables or the int16 matrix. half: those limits hold (the caller asks for the
-// compact layout, or the gather tables do not fit).
+// compact layout, or the gather tables do not fit). rp: with RP records.
 enum SearchKind { SEARCH_TABLES = 0, SEARCH_HALF, SEARCH_CARRY32, SEARCH_CARRY16 };
+// Items of the full evaluation: relocations of two missions, swaps.
+__host__ __device__ inline int64_t search_items(int64_t M, int64_t V) {
+  return (M + V) * ((M + 1) / 2) + M * (M - 1) / 2;
+}
+
 __host__ __device__ inline int pick_search(int M, int V, int L, int nt, bool dl, int ctas, int nwarps, int tenure,
-                                           bool compact, bool half, int limit_words, Layout* out) {
-  const int64_t m = M, items = (m + V) * ((m + 1) / 2) + m * (m - 1) / 2;
-  if (tenure <= kMaxCarryTenure && items > 32ll * kCarryChunks * ctas * nwarps) {
+                                           bool compact, bool half, bool rp, int limit_words, Layout* out) {
+  if (tenure <= kMaxCarryTenure && search_items(M, V) > 32ll * kCarryChunks * ctas * nwarps) {
     if (!compact) {
       *out = make_carry_layout(M, V, L, nt, dl, false, half, ctas, nwarps, tenure);
       if (out->total <= limit_words) return SEARCH_CARRY32;
@@ -246,8 +257,19 @@ __host__ __device__ inline int pick_search(int M, int V, int L, int nt, bool dl,
       if (out->total <= limit_words) return SEARCH_CARRY16;
     }
   }
-  *out = make_layout(M, V, L, nt, half);
+  *out = make_layout(M, V, L, nt, half, rp);
   return half ? SEARCH_HALF : SEARCH_TABLES;
+}
+
+// Whether the full evaluation of a batch or a request takes RP records, relocations of four
+// missions and a pass of their own for neighbours: from 4 chunks of 32 items a warp on, where
+// issue bounds it. Below, pairs without them are faster, since the records cost a barrier
+// (20 missions, 256 threads, 1.7 chunks: 1.8 against 2.2 us an iteration); above, with them
+// (1,024 instances of 100 missions on 2 vehicles, 40 chunks: 49 against 57 us; of 200 210
+// against 248). The line at 3, 4 or 6: between 4 and 6 chunks 0.5 to 1.5 % in favour of 4.
+constexpr int kQuadChunks = 4;
+__host__ __device__ inline bool takes_quads(int M, int V, int ctas, int nwarps) {
+  return search_items(M, V) > 32ll * kQuadChunks * ctas * nwarps;
 }
 
 // ------------------------------------------------------------------ parameters -----
@@ -468,6 +490,7 @@ struct State {  // the per-node records (see the layout notes)
   __device__ __forceinline__ int4* d4() const { return reinterpret_cast<int4*>(g_smem + base + 10 * np); }
   __device__ __forceinline__ int32_t* prv() const { return g_smem + base + 14 * np; }
   __device__ __forceinline__ int32_t* fb() const { return g_smem + base + 15 * np; }
+  __device__ __forceinline__ int32_t* rp() const { return g_smem + base + 15 * np + vp; }
   __device__ __forceinline__ int32_t& nv(int t) const { return g_smem[base + 2 * t]; }
 };
 
@@ -514,7 +537,7 @@ __device__ inline Smem carve(const Layout& y) {
 }
 
 // misc slots
-enum { MISC_BAD = 0, MISC_MAXT, MISC_Z0, MISC_GREEDY_FAIL, MISC_CSR_BAD, MISC_STAGE_FAIL, MISC_STOP };
+enum { MISC_BAD = 0, MISC_MAXT, MISC_Z0, MISC_GREEDY_FAIL, MISC_CSR_BAD, MISC_STAGE_FAIL, MISC_STOP, MISC_VA, MISC_VB };
 
 struct Ctx {  // per-launch constants every thread keeps in registers
   int M, V, N, L, Mp, cap, horizon, lam;
@@ -562,6 +585,35 @@ struct Tab {
       return make_int2(t16((tyl + e.x) * Ls + col), t16((tyl + e.y) * Ls + col));
     }
     return *reinterpret_cast<const int2*>(g_smem + B + r + m0);
+  }
+  // Entries of missions m0 .. m0 + 3 (m0 a multiple of 4), by 128-bit loads.
+  __device__ __forceinline__ int4 a4(int r, int m0) const {
+    if (BIG) {
+      const int4 s = *reinterpret_cast<const int4*>(g_smem + sloc + m0);
+      const int4 cm = *reinterpret_cast<const int4*>(g_smem + cmat + (r >= L ? Mp : 0) + m0);
+      const int base = r * Ls;
+      return make_int4(t16(base + s.x) + cm.x, t16(base + s.y) + cm.y, t16(base + s.z) + cm.z,
+                       t16(base + s.w) + cm.w);
+    }
+    return *reinterpret_cast<const int4*>(g_smem + A + r + m0);
+  }
+  __device__ __forceinline__ int4 b4(int r, int m0) const {
+    if (BIG) {
+      const int tyl = r >= L ? L : 0;
+      const int4 e = *reinterpret_cast<const int4*>(g_smem + eloc + m0);
+      const int col = r - tyl;
+      return make_int4(t16((tyl + e.x) * Ls + col), t16((tyl + e.y) * Ls + col), t16((tyl + e.z) * Ls + col),
+                       t16((tyl + e.w) * Ls + col));
+    }
+    return *reinterpret_cast<const int4*>(g_smem + B + r + m0);
+  }
+  __device__ __forceinline__ int4 tabu4(int v, int m0) const {
+    if (BIG) {
+      const short4 w = *reinterpret_cast<const short4*>(reinterpret_cast<const int16_t*>(g_smem + tabu_off) +
+                                                         v * Mp + m0);
+      return make_int4(w.x, w.y, w.z, w.w);
+    }
+    return *reinterpret_cast<const int4*>(g_smem + tabu_off + v * Mp + m0);
   }
   __device__ __forceinline__ int tabu(int v, int m) const {
     if (BIG) return reinterpret_cast<const int16_t*>(g_smem + tabu_off)[v * Mp + m];
@@ -642,38 +694,54 @@ __device__ __forceinline__ void write_records(const Smem& sm, const Tab<BIG>& tb
   }
 }
 
+// The RP record of a mission: rem its removal delta, fm its route's flight minus the cap.
+template <bool PEN>
+__device__ __forceinline__ int source_part(const Ctx& c, int rem, int fm) {
+  return PEN ? rem + c.lam * (pos0(fm + rem) - pos0(fm)) : (fm + rem <= 0 ? 1 : 0);
+}
+
 __device__ __forceinline__ uint8_t move_flags(bool feas, bool tabu, bool asp, bool adm) {
   return static_cast<uint8_t>((feas ? 1 : 0) | (tabu ? 2 : 0) | (asp ? 4 : 0) | (adm ? 8 : 0));
 }
 
 // Relocation R(m, y): take m out, put it immediately before node y. The inputs are
-// already loaded: m's node word and removal delta, the gap record g of y, the
+// already loaded: m's node word, removal delta and RP record, the gap record g of y, the
 // table entries a = A[row of prev(y)][m], b = B[row of y][m], y's vehicle slack fy and
 // the tabu stamp of (m, vehicle of y). zrel = z_best - Z, so the move aspires when
 // delta < zrel (Z + delta < z_best). An admissible move's key replaces acc when smaller.
 // HELI: the instance has heli-only missions (else the compatibility test is always true).
-template <bool PEN, bool DL, bool DEBUG, bool HELI>
+template <bool PEN, bool DL, bool DEBUG, bool RP, bool HELI>
 __device__ __forceinline__ void reloc_one(const Smem& sm, const State& S, const Ctx& c, int y, int m, int nvm,
-                                          int rem, const int4& g, int a, int b, int fy, int stamp, int it,
+                                          int rem, int rp, const int4& g, int a, int b, int fy, int stamp, int it,
                                           int zrel, const KParams& P, uint64_t& acc) {
-  const bool valid = (y != m) & (y != nv_next(nvm));
+  const bool valid = RP ? (y != m) && (y != nv_next(nvm)) : (y != m) & (y != nv_next(nvm));
   const int vm = nv_veh(nvm), vy = nv_veh(g.w);
   const int ins = a + b - g.z;
   const int d = rem + ins;
-  // Same route: one flight changes by d. Different routes: the source's flight by rem,
-  // the target's by ins. Both are computed and selected, so lanes never diverge.
+  // Same route: one flight changes by d. Different routes: the source's flight by rem
+  // (its part of the delta is m's RP record where kept), the target's by ins. Both are
+  // computed and selected, so lanes never diverge.
   const bool same = vm == vy;
   int delta;
   bool feas;
-  const int fm = S.fb()[vm];
+  const int fm = RP ? 0 : S.fb()[vm];
   int4 dy = make_int4(0, 0, 0, 0);
   int w = 0, leave = 1;
-  if (DL) {
+  if (DL && !RP) {
     dy = S.d4()[y];
     w = sm.wm[m];
     leave = S.d4()[m].w;
   }
-  if (PEN) {
+  if (RP) {
+    const int grow = same ? d : ins;  // change of the target route's flight
+    if (PEN) {
+      delta = (same ? d : rp + ins) + c.lam * (pos0(fy + grow) - pos0(fy));
+      feas = true;
+    } else {
+      delta = d;
+      feas = (fy + grow <= 0) && (same || rp != 0);
+    }
+  } else if (PEN) {
     const int pen = same ? pos0(fy + d) : pos0(fm + rem) - pos0(fm) + pos0(fy + ins);
     delta = d + c.lam * (pen - pos0(fy));
     feas = true;
@@ -681,11 +749,20 @@ __device__ __forceinline__ void reloc_one(const Smem& sm, const State& S, const 
     delta = d;
     feas = same ? (fy + d <= 0) : ((fm + rem <= 0) & (fy + ins <= 0));
   }
-  if (HELI) feas = feas & !((nvm >> 24) & (g.w >> 23) & 1);  // heli-only m onto a plane
-  if (DL) feas = feas & (dy.x + a <= w) & (w + b <= dy.y) & (leave != 0);
+  // Few items a thread (a chain): no branches. Lists (RP, bound by issue): the first condition
+  // that fails ends an item.
+  const bool barred = HELI && ((nvm >> 24) & (g.w >> 23) & 1);  // heli-only m onto a plane
+  if (HELI) feas = RP ? feas && !barred : feas & !barred;
+  if (DL && RP) {
+    dy = S.d4()[y];
+    w = sm.wm[m];
+    feas = feas && (dy.x + a <= w) && (w + b <= dy.y) && S.d4()[m].w;
+  } else if (DL) {
+    feas = feas & (dy.x + a <= w) & (w + b <= dy.y) & (leave != 0);
+  }
   const bool tabu = stamp >= it;
   const bool asp = delta < zrel;
-  const bool adm = valid & feas & (!tabu | asp);
+  const bool adm = RP ? valid && feas && (!tabu || asp) : valid & feas & (!tabu | asp);
   const uint32_t id = (static_cast<uint32_t>(m) << kIdShift) | static_cast<uint32_t>(y);
   if (DEBUG && valid) {
     const int64_t idx = static_cast<int64_t>(m) * (c.N - 2) + y - (y > m) - (y > nv_next(nvm));
@@ -709,9 +786,33 @@ __device__ __forceinline__ void eval_relocate_pair(const Smem& sm, const Tab<BIG
   const int2 b2 = tb.b2(g.y, m0);
   const int2 st = tb.tabu2(vy, m0);
   const int fy = S.fb()[vy];
-  reloc_one<PEN, DL, DEBUG, HELI>(sm, S, c, y, m0, rr.x, rr.y, g, a2.x, b2.x, fy, st.x, it, zrel, P, acc);
+  reloc_one<PEN, DL, DEBUG, false, HELI>(sm, S, c, y, m0, rr.x, rr.y, 0, g, a2.x, b2.x, fy, st.x, it, zrel, P, acc);
   if (m0 + 1 < c.M)
-    reloc_one<PEN, DL, DEBUG, HELI>(sm, S, c, y, m0 + 1, rr.z, rr.w, g, a2.y, b2.y, fy, st.y, it, zrel, P, acc);
+    reloc_one<PEN, DL, DEBUG, false, HELI>(sm, S, c, y, m0 + 1, rr.z, rr.w, 0, g, a2.y, b2.y, fy, st.y, it, zrel, P, acc);
+}
+
+// Relocations of missions m0 .. m0 + 3 (m0 a multiple of 4) before node y, for the item lists
+// of the batch and serving kernels: y's gap record, vehicle, flight and tabu row serve four
+// moves, and the table rows, records and stamps of the four missions come in 128-bit loads.
+template <bool PEN, bool DL, bool BIG, bool HELI>
+__device__ __forceinline__ void eval_relocate_quad(const Smem& sm, const Tab<BIG>& tb, const State& S, const Ctx& c,
+                                                   int y, int m0, int it, int zrel, const KParams& P, uint64_t& acc) {
+  const int4 r01 = *reinterpret_cast<const int4*>(S.r2() + m0);      // {nv, rem} of m0, m0 + 1
+  const int4 r23 = *reinterpret_cast<const int4*>(S.r2() + m0 + 2);  // and of m0 + 2, m0 + 3
+  const int4 rp = *reinterpret_cast<const int4*>(S.rp() + m0);
+  const int4 g = S.y4()[y];  // A row, B row, leg into y, node word of y
+  const int vy = nv_veh(g.w);
+  const int4 a4 = tb.a4(g.x, m0);
+  const int4 b4 = tb.b4(g.y, m0);
+  const int4 st = tb.tabu4(vy, m0);
+  const int fy = S.fb()[vy];
+  reloc_one<PEN, DL, false, true, HELI>(sm, S, c, y, m0, r01.x, r01.y, rp.x, g, a4.x, b4.x, fy, st.x, it, zrel, P, acc);
+  if (m0 + 1 < c.M)
+    reloc_one<PEN, DL, false, true, HELI>(sm, S, c, y, m0 + 1, r01.z, r01.w, rp.y, g, a4.y, b4.y, fy, st.y, it, zrel, P, acc);
+  if (m0 + 2 < c.M)
+    reloc_one<PEN, DL, false, true, HELI>(sm, S, c, y, m0 + 2, r23.x, r23.y, rp.z, g, a4.z, b4.z, fy, st.z, it, zrel, P, acc);
+  if (m0 + 3 < c.M)
+    reloc_one<PEN, DL, false, true, HELI>(sm, S, c, y, m0 + 3, r23.z, r23.w, rp.w, g, a4.w, b4.w, fy, st.w, it, zrel, P, acc);
 }
 
 // Cost parts of swap S(a, b), each mission taking the other's place: t1 = fly from the
@@ -743,10 +844,28 @@ __device__ __forceinline__ SwapParts swap_parts(const Smem& sm, const Tab<BIG>& 
 }
 
 // Swap S(a, b): the two missions exchange places. Aspiration and the key as in reloc_one.
-template <bool PEN, bool DL, bool DEBUG, bool BIG, bool HELI>
+// FAR: the pass over every pair of the batch and serving kernels, which takes the cost parts
+// of two missions that are not neighbours (no delivery rows, no selects) and leaves
+// neighbouring pairs out; those are the pairs (t, next t) of their neighbour pass.
+// FAR = false handles any pair whole (the single-instance kernel's pass over every pair,
+// and the neighbour pass).
+template <bool PEN, bool DL, bool DEBUG, bool BIG, bool HELI, bool FAR>
 __device__ __forceinline__ void eval_swap(const Smem& sm, const Tab<BIG>& tb, const State& S, const Ctx& c, int a,
                                           int b, int it, int zrel, const KParams& P, uint64_t& acc) {
-  const SwapParts q = swap_parts<BIG>(sm, tb, S, c, a, b);
+  SwapParts q;
+  bool near = false;
+  if (FAR) {
+    q.sa = S.s4()[a];
+    q.sb = S.s4()[b];
+    near = nv_next(q.sa.x) == b || nv_next(q.sb.x) == a;
+    q.adjA = q.adjB = false;
+    q.t1 = tb.a(q.sa.y, b);
+    q.t2 = tb.b(q.sa.z, b);
+    q.t3 = tb.a(q.sb.y, a);
+    q.t4 = tb.b(q.sb.z, a);
+  } else {
+    q = swap_parts<BIG>(sm, tb, S, c, a, b);
+  }
   const int nva = q.sa.x, nvb = q.sb.x;
   const int va = nv_veh(nva), vb = nv_veh(nvb);
   const int da = q.t1 + q.t2 - q.sa.w;
@@ -762,21 +881,34 @@ __device__ __forceinline__ void eval_swap(const Smem& sm, const Tab<BIG>& tb, co
     feas = true;
   } else {
     delta = d;
-    feas = same ? (fa + d <= 0) : ((fa + da <= 0) & (fb + db <= 0));
+    feas = same ? (fa + d <= 0) : FAR ? (fa + da <= 0) && (fb + db <= 0) : ((fa + da <= 0) & (fb + db <= 0));
   }
-  if (HELI) feas = feas & !((((nva >> 24) & (nvb >> 23)) | ((nvb >> 24) & (nva >> 23))) & 1);
-  if (DL) {
-    const int4 xa = S.d4()[a], xb = S.d4()[b];
-    const int wa = sm.wm[a], wb = sm.wm[b];
-    const bool l1 = (q.adjB ? wa : xa.x) + q.t1 <= wb;
-    const bool l2 = q.adjA | (wb + q.t2 <= xa.z);
-    const bool l3 = (q.adjA ? wb : xb.x) + q.t3 <= wa;
-    const bool l4 = q.adjB | (wa + q.t4 <= xb.z);
-    feas = feas & l1 & l2 & l3 & l4;
-  }
-  const bool tabu = (tb.tabu(vb, a) >= it) | (tb.tabu(va, b) >= it);
   const bool asp = delta < zrel;
-  const bool adm = feas & (!tabu | asp);
+  bool tabu, adm;  // with and without branches as in reloc_one
+  const bool barred = HELI && ((((nva >> 24) & (nvb >> 23)) | ((nvb >> 24) & (nva >> 23))) & 1);
+  if (FAR) {
+    if (HELI) feas = feas && !barred;
+    if (DL) {
+      const int4 xa = S.d4()[a], xb = S.d4()[b];
+      const int wa = sm.wm[a], wb = sm.wm[b];
+      feas = feas && xa.x + q.t1 <= wb && wb + q.t2 <= xa.z && xb.x + q.t3 <= wa && wa + q.t4 <= xb.z;
+    }
+    tabu = tb.tabu(vb, a) >= it || tb.tabu(va, b) >= it;
+    adm = !near && feas && (!tabu || asp);
+  } else {
+    if (HELI) feas = feas & !barred;
+    if (DL) {
+      const int4 xa = S.d4()[a], xb = S.d4()[b];
+      const int wa = sm.wm[a], wb = sm.wm[b];
+      const bool l1 = (q.adjB ? wa : xa.x) + q.t1 <= wb;
+      const bool l2 = q.adjA | (wb + q.t2 <= xa.z);
+      const bool l3 = (q.adjA ? wb : xb.x) + q.t3 <= wa;
+      const bool l4 = q.adjB | (wa + q.t4 <= xb.z);
+      feas = feas & l1 & l2 & l3 & l4;
+    }
+    tabu = (tb.tabu(vb, a) >= it) | (tb.tabu(va, b) >= it);
+    adm = feas & (!tabu | asp);
+  }
   const int m1 = a < b ? a : b, m2 = a < b ? b : a;
   const uint32_t id = kSwapBit | (static_cast<uint32_t>(m1) << kIdShift) | static_cast<uint32_t>(m2);
   if (DEBUG) {
@@ -795,14 +927,16 @@ __device__ __forceinline__ void eval_swap(const Smem& sm, const Tab<BIG>& tb, co
 struct ItemCursor {
   int r_y, r_h, s_j, s_row, s_a;  // first relocation item (y, h) and swap item (j, row, a)
   int Gq, Gr, Sq, Sr, G, H, Sn;   // grid stride in both coordinate systems, list sizes
+  int n_k;                        // first item of the neighbour pass (mission t)
 };
 
-template <bool PEN, bool DL, bool DEBUG, bool BIG, bool HELI>
+template <bool PEN, bool DL, bool DEBUG, bool BIG, bool RP, bool HELI>
 __device__ __forceinline__ uint64_t eval_items(const Smem& sm, const Tab<BIG>& tb, const State& S, const Ctx& c,
                                                const ItemCursor& q, int it, int zrel, const KParams& P) {
   uint64_t key = kNoKey;
   for (int y = q.r_y, h = q.r_h; y < c.N;) {
-    eval_relocate_pair<PEN, DL, DEBUG, BIG, HELI>(sm, tb, S, c, y, 2 * h, it, zrel, P, key);
+    if (RP) eval_relocate_quad<PEN, DL, BIG, HELI>(sm, tb, S, c, y, 4 * h, it, zrel, P, key);
+    else eval_relocate_pair<PEN, DL, DEBUG, BIG, HELI>(sm, tb, S, c, y, 2 * h, it, zrel, P, key);
     h += q.Gr;
     y += q.Gq;
     if (h >= q.H) {
@@ -813,12 +947,22 @@ __device__ __forceinline__ uint64_t eval_items(const Smem& sm, const Tab<BIG>& t
   for (int j = q.s_j, row = q.s_row, a = q.s_a; j < q.Sn; j += q.G) {
     int b = a + row + 1;
     if (b >= c.M) b -= c.M;
-    eval_swap<PEN, DL, DEBUG, BIG, HELI>(sm, tb, S, c, a, b, it, zrel, P, key);
+    eval_swap<PEN, DL, DEBUG, BIG, HELI, RP>(sm, tb, S, c, a, b, it, zrel, P, key);
     a += q.Sr;
     row += q.Sq;
     if (a >= c.M) {
       a -= c.M;
       ++row;
+    }
+  }
+  // Swaps of neighbours, t and its successor (the batch and serving kernels only, which
+  // are bound by instruction issue: the pass above then takes the short form of every
+  // pair; the single-instance kernel, bound by the latency of its slowest warp, keeps one
+  // pass over the pairs with the neighbour case inside).
+  if (RP) {
+    for (int t = q.n_k; t < c.M; t += q.G) {
+      const int u = nv_next(S.nv(t));
+      if (u < c.M) eval_swap<PEN, DL, DEBUG, BIG, HELI, false>(sm, tb, S, c, t, u, it, zrel, P, key);
     }
   }
   return key;
@@ -884,7 +1028,7 @@ __device__ __forceinline__ uint64_t eval_narrow(const Smem& sm, const Tab<BIG>& 
     const int vy = nv_veh(g.w);
     const int a = tb.a(g.x, m), b = tb.b(g.y, m), stamp = tb.tabu(vy, m), fy = S.fb()[vy];
     uint64_t key = kNoKey;
-    reloc_one<PEN, DL, false, true>(sm, S, c, y, m, r.x, r.y, g, a, b, fy, stamp, it, zrel, P, key);
+    reloc_one<PEN, DL, false, false, true>(sm, S, c, y, m, r.x, r.y, 0, g, a, b, fy, stamp, it, zrel, P, key);
     return n.live ? key : kNoKey;
   }
   if (n.kind == 3) {
@@ -1095,8 +1239,8 @@ __device__ __forceinline__ bool stage_matrix16(const KParams& P, const Layout& l
 
 // Prologue 1 of a search: static per-mission and per-node data, range-checked (this
 // thread's share; the flag says whether an entry was out of range). The caller zeroes the
-// misc words first and synchronises afterwards.
-__device__ __forceinline__ int load_statics(const KParams& P, const Smem& sm, int Mp, int& any_heli) {
+// misc words first and synchronises afterwards. nodes: entries of the location arrays.
+__device__ __forceinline__ int load_statics(const KParams& P, const Smem& sm, int Mp, int nodes, int& any_heli) {
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int M = P.M, V = P.V, N = P.M + P.V, L = P.L, nt = P.nt;
   int bad = 0;
@@ -1124,7 +1268,7 @@ __device__ __forceinline__ int load_statics(const KParams& P, const Smem& sm, in
     sm.tyl[v] = ty * L;
     sm.tym[v] = ty * Mp;
   }
-  for (int i = N + tid; i < round_up(N + 1, 4); i += nthr) {  // padding read by pairs of missions
+  for (int i = N + tid; i < nodes; i += nthr) {  // padding read by pairs or quads of missions
     sm.eloc[i] = 0;
     sm.sloc[i] = 0;
   }
@@ -1492,7 +1636,7 @@ __device__ __forceinline__ void write_info(int32_t* info, int status, int zbest,
 // the K clusters of C CTAs each (this CTA is `rank` in cluster `cid`), with shared
 // memory laid out by lay. Every CTA holds the whole state and applies every move; CTA 0
 // of cluster 0 writes the outputs.
-template <bool PEN, bool DL, bool DEBUG, bool BIG>
+template <bool PEN, bool DL, bool DEBUG, bool BIG, bool RP>
 __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, const int C, const int rank,
                                           const int K, const int cid) {
   const bool lead = rank == 0 && cid == 0;
@@ -1516,7 +1660,7 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
   if (tid < 16) sm.misc[tid] = 0;
   __syncthreads();
   int any_heli = 0;
-  int bad = load_statics(P, sm, Mp, any_heli);
+  int bad = load_statics(P, sm, Mp, round_up(N + 3, 4), any_heli);
   int maxT = 0;
   if (!BIG) {  // the compact layout checks the matrix while it stages it (prologue 2)
     for (int i = tid; i < nt * L * L; i += nthr) {
@@ -1593,6 +1737,7 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
     const bool ok = start_records<PEN, DL>(sm, tb, S0, c, [&](int t, int nx, int pv, int vw, int f) {
       write_records<PEN, DL, BIG>(sm, tb, S0, c, t, nx, pv, vw);
       if (t >= M) S0.fb()[t - M] = f - c.cap;
+      else if (RP) S0.rp()[t] = source_part<PEN>(c, S0.r2()[t].y, f - c.cap);
     });
     if (!ok) status = ASCHED_E_INFEASIBLE_INIT;
     for (int t = tid; t < N; t += nthr) sm.best[t] = nv_next(S0.nv(t));
@@ -1608,18 +1753,21 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
   if (looped) {
     if (C > 1) cluster_sync_all();
     // Static assignment over the item list [relocation pairs (N * ceil(M/2)) | swaps
-    // (M(M-1)/2)]: chunks of 32 consecutive items go round-robin to (CTA, warp) over the
-    // K * C CTAs of the grid, so every CTA gets an equal share and the lanes of a warp take
-    // consecutive items. A relocation item i is (y, h) = divmod(i, H) for missions 2h and
-    // 2h + 1; a swap item j is (row, a) = divmod(j, M) with b = (a + row + 1) mod M, which
-    // lists every pair a != b once. Coordinates advance by G without dividing.
+    // (M(M-1)/2) | neighbour swaps (M, with RP records only)]: chunks of 32 consecutive items
+    // go round-robin to (CTA, warp) over the K * C CTAs of the grid, so every CTA gets an
+    // equal share and the lanes of a warp take consecutive items. A relocation item i is
+    // (y, h) = divmod(i, H) for missions 2h and 2h + 1 (with RP records for missions 4h ..
+    // 4h + 3); a swap item j is (row, a) = divmod(j, M) with b = (a + row + 1) mod M, which
+    // lists every pair a != b once (with RP records neighbours in a route are left out there,
+    // and a neighbour item t swaps mission t with its successor when that is a mission).
+    // Coordinates advance by G without dividing.
     const int CT = K * C;
     const int G = CT * nthr;
     const int g = lane + 32 * (cid * C + rank + CT * warp);
-    const int H = (M + 1) / 2;  // relocation items per node y
+    const int H = RP ? (M + 3) / 4 : (M + 1) / 2;  // relocation items per node y
     const int Rn = N * H;
     const int Sn = M * (M - 1) / 2;
-    int r_y = N, r_h = 0, s_j = Sn, s_row = 0, s_a = 0, Gq = 0, Gr = 0, Sq = 0, Sr = 0;
+    int r_y = N, r_h = 0, s_j = Sn, s_row = 0, s_a = 0, Gq = 0, Gr = 0, Sq = 0, Sr = 0, n_k = M;
     if (M > 0) {
       Gq = G / H;
       Gr = G - Gq * H;
@@ -1635,8 +1783,10 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
         s_row = s_j / M;
         s_a = s_j - s_row * M;
       }
+      const int k2 = g < Rn + Sn ? (Rn + Sn - g + G - 1) / G : 0;  // items before the neighbour pass
+      n_k = g + k2 * G - (Rn + Sn);
     }
-    const ItemCursor cursor{r_y, r_h, s_j, s_row, s_a, Gq, Gr, Sq, Sr, G, H, Sn};
+    const ItemCursor cursor{r_y, r_h, s_j, s_row, s_a, Gq, Gr, Sq, Sr, G, H, Sn, n_k};
     // One item a thread, with relocations singly if they fit, else two missions an item; or two.
     // Measured on single searches, narrow against the general lists: 10 missions (6 warps,
     // pairs) 291 -> 209 us for 200 iterations; 24 missions of the paper's fleet (64 warps, one
@@ -1644,7 +1794,7 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
     // the copies. Up to four rounds lost: 100 missions (3.6 rounds) 8.7 ms against 7.7 ms.
     const int64_t threads32 = static_cast<int64_t>(CT) * nwarps;
     const int64_t single = narrow_chunks(M, V, false), paired = narrow_chunks(M, V, true);
-    const bool narrow = !DEBUG && (single <= kNarrowItems * threads32);
+    const bool narrow = !DEBUG && !RP && (single <= kNarrowItems * threads32);
     const bool pairs = single > threads32 && paired <= threads32;
     uint32_t item[kNarrowItems];
 #pragma unroll
@@ -1672,8 +1822,8 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
           i1 = 0u;
         }
       } else {
-        key = c.heli ? eval_items<PEN, DL, DEBUG, BIG, true>(sm, tb, S, c, cursor, it_eval, zrel, P)
-                     : eval_items<PEN, DL, DEBUG, BIG, false>(sm, tb, S, c, cursor, it_eval, zrel, P);
+        key = c.heli ? eval_items<PEN, DL, DEBUG, BIG, RP, true>(sm, tb, S, c, cursor, it_eval, zrel, P)
+                     : eval_items<PEN, DL, DEBUG, BIG, RP, false>(sm, tb, S, c, cursor, it_eval, zrel, P);
       }
       if (copy_best) {
         for (int t = tid; t < N; t += nthr) sm.best[t] = nv_next(S.nv(t));
@@ -1733,6 +1883,10 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
         } else if (warp <= wstamp) {
           const int va = nv_veh(S.nv(n1)), vb = nv_veh(S.nv(n2));
           if (warp == 1) {
+            if (RP && lane == 0) {
+              sm.misc[MISC_VA] = moved ? va : -1;
+              sm.misc[MISC_VB] = moved ? vb : -1;
+            }
             const int f = moved ? moved_flight<BIG>(sm, tb, S, c, id, lane == 0) : 0;
             named_arrive(1, readers);
             if (moved && (lane == 0 || (lane == 1 && va != vb))) S.fb()[lane == 0 ? va : vb] = f - c.cap;
@@ -1759,6 +1913,15 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
         status = sm.misc[MISC_STOP];
         break;
       }
+      if (RP) {  // the RP records of the changed routes, from their new flights
+        const int va = sm.misc[MISC_VA], vb = sm.misc[MISC_VB];
+        for (int t = tid; t < M; t += nthr) {
+          const int2 r = S0.r2()[t];
+          const int v = nv_veh(r.x);
+          if (v == va || v == vb) S0.rp()[t] = source_part<PEN>(c, r.y, S0.fb()[v]);
+        }
+        __syncthreads();
+      }
     }
     if (copy_best) {
       for (int t = tid; t < N; t += nthr) sm.best[t] = nv_next(S0.nv(t));
@@ -1771,12 +1934,6 @@ __device__ __forceinline__ void solve_one(const KParams& P, const Layout& lay, c
   if (lead && tid == 0 && P.info) write_info(P.info, status, zbest, best_it, sm.misc[MISC_Z0], Z, it);
   // No CTA may leave while a peer can still write into its shared memory.
   if (C > 1 && looped) cluster_sync_unaligned();
-}
-
-// The full evaluation as a call, for kernels that carry several searches.
-template <bool PEN, bool DL, bool BIG>
-__device__ __noinline__ void solve_full(const KParams& P, const Layout& lay, int C, int rank, int K, int cid) {
-  solve_one<PEN, DL, false, BIG>(P, lay, C, rank, K, cid);
 }
 
 #include "carry.cuh"
