@@ -4,11 +4,11 @@
 #include "kernels.h"
 #include "nvtx_range.h"
 
+#include <math.h>
+
 namespace {
 
 // ------------------------------------------------------------------ host side ------
-
-constexpr int kBatchThreads = 256;  // per CTA of a batch, two CTAs per SM
 
 // Shared-memory layout for an instance: the gather tables when they fit, else the
 // int16 matrix (whose stamps limit iterations + tenure to 32,767). What a call accepts
@@ -288,6 +288,70 @@ int launch(const asched_instance* inst, const asched_params* p, bool debug, KPar
   return ASCHED_OK;
 }
 
+// One way to run a batch: CTAs of `threads`, per_sm of them on an SM at once.
+struct BatchForm {
+  int threads, per_sm;
+  int limit_words;  // shared memory by which each instance's form is chosen
+  int words;        // the most any of them takes
+  int places;       // instances (CTAs or clusters) at once
+  double time;      // estimate of an iteration of all
+};
+
+// The estimate, in items of the full evaluation (see carry_cost): an iteration of an instance takes
+// 208 + c r / (C e(r W)) with r CTAs of W warps on its SM, e(w) = 24 w / (w + 8) the items an SM gets
+// done with w warps (200 missions on 3 vehicles by the full evaluation: 64 threads 83 us, 128 42.4,
+// 256 25.1, 512 18.4; 208 items are 1.4 us). The longest start first. A batch takes the longest,
+// whose SM is its own once its neighbours are through, or the sum over all places, or, with more
+// instances than places, those that have to share one. Over 48 batches of 100 to 1,024 instances,
+// equal and mixed, mostly within 15 %, and the choice within 3 % of the better one.
+int batch_form(const asched_batch* bt, const asched_params* p, int C, int sms, int table_words, BatchForm* f) {
+  const bool dl = bt->deadline != nullptr, compact = (p->flags & ASCHED_COMPACT_LAYOUT) != 0;
+  const int W = f->threads / 32, r = f->per_sm, B = bt->n_instances;
+  const auto per_item = [&](int k) { return k * (k * W + 8.0) / (24.0 * k * W * C); };  // with k CTAs on the SM
+  constexpr int kFixed = 208, kBins = 16 * 24;  // 16 per octave of an instance's items
+  int bins[kBins] = {};
+  double sum = 0.0, most = 0.0;
+  f->words = 0;
+  for (int b = 0; b < B; ++b) {
+    const int L = bt->h_loc_off[b + 1] - bt->h_loc_off[b], V = bt->h_veh_off[b + 1] - bt->h_veh_off[b],
+              M = bt->h_mis_off[b + 1] - bt->h_mis_off[b];
+    const bool half = compact || make_layout(M, V, L, bt->n_types, false, true).total > table_words;
+    Layout lay;
+    const int kind = pick_search(M, V, L, bt->n_types, dl, C, W, p->tenure, compact, half, true, f->limit_words, &lay);
+    if (lay.total > f->limit_words) return ASCHED_E_TOO_LARGE;
+    if (lay.total > f->words) f->words = lay.total;
+    const bool carried = kind == SEARCH_CARRY32 || kind == SEARCH_CARRY16;
+    const double c = 1.0 + (carried ? 0.25 * carry_cost(M, V, dl, C, W) : static_cast<double>(search_items(M, V)));
+    sum += c;
+    most = c > most ? c : most;
+    const int bin = static_cast<int>(16.0 * log2(c));
+    ++bins[bin < kBins ? bin : kBins - 1];
+  }
+  const auto nth = [&](int n) {  // items of the n-th longest instance, n < B
+    int bin = kBins - 1;
+    for (int k = bins[bin]; k <= n; k += bins[bin]) --bin;
+    return exp2((bin + 0.5) / 16.0);
+  };
+  f->places = sms * r / C;
+  if (C > 1) {
+    const int rc = active_clusters(asched_kernels::batch(p->cap_mode == ASCHED_PENALTY, dl, true), C, f->threads,
+                                   f->words * 4, &f->places);
+    if (rc != ASCHED_OK) return rc;
+    if (f->places < 1) return ASCHED_E_TOO_LARGE;
+  }
+  const int sets = (f->places + r - 1) / r;  // SMs, or groups of C of them
+  f->time = (kFixed * static_cast<double>(B) + sum * per_item(r)) / f->places;
+  double longest = kFixed + most * per_item(1);
+  if (B <= f->places && B > sets) longest += nth(sets) * (per_item(r) - per_item(1));
+  for (int64_t j = 1; j * f->places < B; ++j) {  // of j places + 1 instances some place gets j + 1
+    const int n = static_cast<int>(j) * f->places, rest = (B - n + sets - 1) / sets;
+    const double all = (j + 1) * kFixed + nth(n) * (j * per_item(r) + per_item(rest < r ? rest : r));
+    longest = all > longest ? all : longest;
+  }
+  f->time = longest > f->time ? longest : f->time;
+  return ASCHED_OK;
+}
+
 int launch_batch(const asched_batch* bt, const asched_params* p, const asched_batch_result* out,
                  void* workspace, size_t ws_bytes, void* stream) {
   if (!bt || !p || !out) return ASCHED_E_INVALID;
@@ -305,8 +369,6 @@ int launch_batch(const asched_batch* bt, const asched_params* p, const asched_ba
   const int limit_words = (limit - 64) / 4;
   // CTAs per instance: 1 (one persistent CTA per SM slot) or a cluster of C CTAs
   const int C = p->cluster_size > 1 ? p->cluster_size : 1;
-  const int threads = p->block_threads ? p->block_threads : kBatchThreads;
-  int max_words = 0;
   asched_instance one = {};
   one.n_types = bt->n_types;
   one.duty_cap = 0;
@@ -315,16 +377,40 @@ int launch_batch(const asched_batch* bt, const asched_params* p, const asched_ba
     one.n_loc = bt->h_loc_off[b + 1] - bt->h_loc_off[b];
     one.n_vehicles = bt->h_veh_off[b + 1] - bt->h_veh_off[b];
     one.n_missions = bt->h_mis_off[b + 1] - bt->h_mis_off[b];
-    int rc = check_sizes(&one, p);
-    if (rc != ASCHED_OK) return rc;
+    int bad = check_sizes(&one, p);
+    if (bad != ASCHED_OK) return bad;
     Layout lay;
-    rc = choose_layout(one.n_missions, one.n_vehicles, one.n_loc, one.n_types, p, limit, true, &lay);
-    if (rc != ASCHED_OK) return rc;
-    pick_search(one.n_missions, one.n_vehicles, one.n_loc, one.n_types, bt->deadline != nullptr, C, threads / 32,
-                p->tenure, (p->flags & ASCHED_COMPACT_LAYOUT) != 0, lay.big, true, limit_words, &lay);
-    if (lay.total > max_words) max_words = lay.total;
+    bad = choose_layout(one.n_missions, one.n_vehicles, one.n_loc, one.n_types, p, limit, true, &lay);
+    if (bad != ASCHED_OK) return bad;
   }
-  const int64_t bytes = static_cast<int64_t>(max_words) * 4;
+  int dev = 0, sms = 0, sm_bytes = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return ASCHED_E_CUDA;
+  }
+  // The block: 512 threads one per SM, or, with more instances than that has places for, 256 threads
+  // two per SM, by the estimate; a caller's block as many per SM as the estimate finds best. Two per
+  // SM get more done (250 iterations of 304 instances, us each: 40 missions on 8 vehicles 3.1
+  // against 4.4, 100 on 20 7.1 against 9.0, 200 on 30 13.2 against 15.4) and share 228 KB, where the
+  // tables of a large instance with few vehicles do not fit and the carried form is slower (200 on
+  // 3: 38.9 against 36.4); one finishes the longest instances of a mixed batch sooner (512 of 10 to
+  // 200 missions on 3 to 30 vehicles 16.2 against 20.0, 1,024 of them 31.5 against 27.0).
+  const int own = p->block_threads;
+  BatchForm form = {own ? own : kMaxThreads, 1, limit_words, 0, 0, 0.0};
+  int rc = batch_form(bt, p, C, sms, limit_words, &form);
+  if (rc != ASCHED_OK) return rc;
+  const int per_sm_most = own ? kMaxThreads / own : 2;
+  for (int r = 2, places = form.places; r <= per_sm_most && B > places; r *= 2) {
+    BatchForm f = {own ? own : kMaxThreads / r, r, (sm_bytes / r - 1024 - 64) / 4, 0, 0, 0.0};
+    if (f.limit_words > limit_words) f.limit_words = limit_words;
+    if (batch_form(bt, p, C, sms, limit_words, &f) != ASCHED_OK) break;
+    places = f.places;
+    if (f.time < form.time) form = f;
+  }
+  const int threads = form.threads;
+  const int64_t bytes = static_cast<int64_t>(form.words) * 4;
   const bool pen = p->cap_mode == ASCHED_PENALTY;
   const bool dl = bt->deadline != nullptr;
   void* fn = asched_kernels::batch(pen, dl, C > 1);
@@ -334,16 +420,13 @@ int launch_batch(const asched_batch* bt, const asched_params* p, const asched_ba
   int grid = 0;
   if (C > 1) {
     int n = 0;
-    const int rc = active_clusters(fn, C, threads, static_cast<int>(bytes), &n);
+    rc = active_clusters(fn, C, threads, static_cast<int>(bytes), &n);
     if (rc != ASCHED_OK) return rc;
     if (n < 1) return ASCHED_E_TOO_LARGE;
     grid = (B < n ? B : n) * C;
   } else {
-    int dev = 0, sms = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, static_cast<size_t>(bytes)) !=
-            cudaSuccess) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, static_cast<size_t>(bytes)) != cudaSuccess) {
       (void)cudaGetLastError();
       return ASCHED_E_CUDA;
     }
@@ -358,7 +441,8 @@ int launch_batch(const asched_batch* bt, const asched_params* p, const asched_ba
   q.run.cluster = C;
   q.run.timeout_ns = p->timeout_ns > 0 ? p->timeout_ns : kDefaultTimeoutNs;
   q.B = B;
-  q.limit_words = limit_words;
+  q.table_words = limit_words;
+  q.limit_words = form.limit_words;
   q.compact = (p->flags & ASCHED_COMPACT_LAYOUT) ? 1 : 0;
   q.loc_off = bt->loc_off;
   q.veh_off = bt->veh_off;

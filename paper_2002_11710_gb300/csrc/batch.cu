@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) tabu_batch_kernel(const __grid
     P.out_flight = Q.out_flight + vo;
     P.out_over = Q.out_over + vo;
     P.info = Q.info + static_cast<int64_t>(b) * ASCHED_INFO_LEN;
-    search_instance<PEN, DL>(P, C, rank, Q.compact != 0, Q.limit_words, Q.limit_words);
+    search_instance<PEN, DL>(P, C, rank, Q.compact != 0, Q.table_words, Q.limit_words);
     __syncthreads();  // the next instance's prologue reuses shared memory
   }
 }

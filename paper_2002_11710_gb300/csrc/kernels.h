@@ -17,7 +17,8 @@ __host__ __device__ inline int64_t moves_of(int64_t M, int64_t V) { return M * (
 struct BParams {
   KParams run;  // tenure, iterations, lambda, nt, timeout; no instance pointers
   int32_t B;
-  int32_t limit_words;  // shared memory a CTA may use: the layout rule's limit (see pick_search)
+  int32_t table_words;  // gather tables up to this size do without the int16 limits
+  int32_t limit_words;  // shared memory of a CTA by which the form of a search is chosen (see pick_search)
   int32_t compact;      // always take the int16 matrix
   const int32_t* loc_off;
   const int32_t* veh_off;

@@ -143,7 +143,6 @@ __host__ __device__ inline Layout make_layout(int M, int V, int L, int nt, bool 
 // Layouts with carried move values (carry.cuh): the matrix itself (int32 with an odd row
 // stride, or int16 as above) at the start, the records, and the tables of one CTA's slice
 // of the missions.
-constexpr int kCarryChunks = 6;
 constexpr int kMaxCarryTenure = 512;  // ring of moves; longer tenures take the full evaluation
 __host__ __device__ inline Layout make_carry_layout(int M, int V, int L, int nt, bool dl, bool t16, bool half,
                                                     int ctas, int nwarps, int tenure) {
@@ -235,19 +234,50 @@ __host__ __device__ inline Layout make_carry_layout(int M, int V, int L, int nt,
   return y;
 }
 
-// The layout of a search: carried move values when they fit (with the int32 matrix, or, where
-// the limits of the int16 matrix hold anyway, the int16 one), else the full evaluation with
-// the gather tables or the int16 matrix. half: those limits hold (the caller asks for the
-// compact layout, or the gather tables do not fit). rp: with RP records.
-enum SearchKind { SEARCH_TABLES = 0, SEARCH_HALF, SEARCH_CARRY32, SEARCH_CARRY16 };
 // Items of the full evaluation: relocations of two missions, swaps.
 __host__ __device__ inline int64_t search_items(int64_t M, int64_t V) {
   return (M + V) * ((M + 1) / 2) + M * (M - 1) / 2;
 }
 
+// Whether carried move values are faster than the full evaluation, on one cluster. Full: its
+// items. Carried, in the same unit (all times four): a fixed part per warp for the chain of
+// table updates; P, the pairs of a node of the two changed routes and a mission (two routes of
+// average length; with one vehicle its only one), each of which takes both sides of a swap; and
+// V M, the entries that are scanned. With few vehicles P is most of the neighbourhood: that is
+// where the line lies. On clusters a pair costs more, since every CTA keeps all nodes' records
+// for a slice of the missions. Arrive-by times lengthen the full evaluation more. Fitted to both
+// sides at 20 to 300 missions, 1 to 50 vehicles, 1 to 1,024 instances, 64 to 512 threads, 1 to 16
+// CTAs; the rule's choice is on average 0.2 to 0.7 % slower than the better side. us an
+// iteration, full / carried:
+//   one instance, 512 threads:  200 missions on 1 vehicle 17.5 / 34.3, on 4 18.9 / 19.4, on 8
+//     18.9 / 11.5; 100 on 4 6.3 / 8.6, on 8 6.4 / 5.5; 40 on 8 2.7 / 3.4
+//   1,024 instances, 256 threads:  200 on 3 208 / 194, on 12 207 / 88; 100 on 4 48.5 / 68.6, on
+//     8 48.6 / 48.1, on 20 50.1 / 37.3; 60 on 12 27.7 / 26.1; 40 on 8 19.7 / 24.0
+//   a cluster of 8 CTAs of 256 threads:  200 on 12 5.8 / 6.3, on 20 6.0 / 5.5; 300 on 20
+//     11.8 / 9.1; 100 on 20 3.2 / 3.7
+__host__ __device__ inline int64_t carry_cost(int64_t M, int64_t V, bool dl, int64_t ctas, int64_t nwarps) {
+  const int64_t pairs = V == 1 ? (M + 1) * M : 2 * M * (M + V) / V, entries = V * M;
+  if (ctas == 1) {
+    const int64_t rest = pairs + entries < 40 * M ? pairs + entries : 40 * M;
+    return dl ? 400 * nwarps + 5 * pairs + 2 * entries : 600 * nwarps + 6 * pairs + 4 * rest;
+  }
+  const int64_t f = ctas <= 4 ? 7 : 12;
+  return dl ? 400 * ctas * nwarps + f * pairs + 2 * entries : 600 * ctas * nwarps + 2 * f * pairs + 4 * entries;
+}
+__host__ __device__ inline bool carry_pays(int64_t M, int64_t V, bool dl, int64_t ctas, int64_t nwarps) {
+  return 4 * search_items(M, V) > carry_cost(M, V, dl, ctas, nwarps);
+}
+
+// The layout of a search: carried move values where they fit limit_words (with the int32 matrix,
+// or, where the limits of the int16 matrix hold anyway, the int16 one) and pay, or the full
+// evaluation does not fit; else the full evaluation with the gather tables or the int16 matrix,
+// whatever it takes. half: those limits hold (the caller asks for the
+// compact layout, or the gather tables do not fit). rp: with RP records.
+enum SearchKind { SEARCH_TABLES = 0, SEARCH_HALF, SEARCH_CARRY32, SEARCH_CARRY16 };
 __host__ __device__ inline int pick_search(int M, int V, int L, int nt, bool dl, int ctas, int nwarps, int tenure,
                                            bool compact, bool half, bool rp, int limit_words, Layout* out) {
-  if (tenure <= kMaxCarryTenure && search_items(M, V) > 32ll * kCarryChunks * ctas * nwarps) {
+  const Layout full = make_layout(M, V, L, nt, half, rp);
+  if (tenure <= kMaxCarryTenure && (carry_pays(M, V, dl, ctas, nwarps) || full.total > limit_words)) {
     if (!compact) {
       *out = make_carry_layout(M, V, L, nt, dl, false, half, ctas, nwarps, tenure);
       if (out->total <= limit_words) return SEARCH_CARRY32;
@@ -257,7 +287,7 @@ __host__ __device__ inline int pick_search(int M, int V, int L, int nt, bool dl,
       if (out->total <= limit_words) return SEARCH_CARRY16;
     }
   }
-  *out = make_layout(M, V, L, nt, half, rp);
+  *out = full;
   return half ? SEARCH_HALF : SEARCH_TABLES;
 }
 
