@@ -84,13 +84,17 @@ struct Inst {
   WarpLayout y;
 };
 
-// The time at offset o of the node-to-node times: end node row, start node column.
+// The time at offset o of the node-to-node times: end node row, start node column. From the
+// matrix itself (H false) rows are kWideRow apart, so that an offset splits without a division,
+// and their matrix rows lie where the times would (4,096 instances of 36 nodes, Algorithm 3: 329 us;
+// with divisions 474, one CTA of 32 threads with linked lists 371).
+constexpr int kWideRow = 64;
+static_assert(kWideRow >= asched_kernels::kWarpNodes, "a column per node");
 template <bool H>
 __device__ __forceinline__ int time_at(const Inst& s, int o) {
   if (H) return reinterpret_cast<const int16_t*>(g_warp + s.y.times)[o];
-  const int r = o / s.y.row, col = o - r * s.y.row;
-  const int ty = r / s.N, e = r - ty * s.N;
-  return __ldg(s.T + (static_cast<int64_t>(ty) * s.L + word(s.y.eloc, e)) * s.L + word(s.y.sloc, col));
+  const int64_t r = word(s.y.times, o / kWideRow);  // offsets are at least 0
+  return __ldg(s.T + r * s.L + word(s.y.sloc, o % kWideRow));
 }
 
 // The register of position p (any lane's) of all positions x.
@@ -116,7 +120,7 @@ __device__ __forceinline__ int first_pos(bool x0, bool x1) {
 template <bool PEN, bool DL, bool TABU, bool H>
 __device__ __forceinline__ void search(const SwParams& Q, const Inst& s) {
   const int lane = threadIdx.x & 31;
-  const int M = s.M, V = s.V, N = s.N, cap = s.cap, lam = s.lam, row = s.y.row;
+  const int M = s.M, V = s.V, N = s.N, cap = s.cap, lam = s.lam, row = H ? s.y.row : kWideRow;
   const bool two = N > 32;  // both registers are in use
   const int4* const mis = reinterpret_cast<const int4*>(g_warp + s.y.mis);
   // ---- positions: node | vehicle << 8, and their records
@@ -666,6 +670,8 @@ __global__ void __launch_bounds__(32, 20) sweep_warp_kernel(const __grid_constan
       }
     }
   }
+  if (!half)  // matrix rows of the end nodes, by layer
+    for (int x = lane; x < nt * N; x += 32) word(s.y.times, x) = x < N ? word(s.y.eloc, x) : L + word(s.y.eloc, x - N);
   if (TABU)
     for (int x = lane; x < M * V; x += 32) word(s.y.tabu, x) = -1;
   __syncwarp();
