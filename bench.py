@@ -57,9 +57,11 @@ WORKLOADS = {
 OPS_RELOCATE, OPS_SWAP = 20, 30
 GATHERS_RELOCATE, GATHERS_SWAP = 3, 6
 # DRAM bytes (read + write) per launch of the headline kernel from one ncu capture,
-# keyed by the first 16 hex digits of the SHA-256 of csrc/asched.cu it was taken on;
-# any other source reports traffic as null.
-TRAFFIC_BYTES = {"047155f641486d20": 916224}  # ncu launch list of the large-instance bench, mean of 12 launches
+# keyed by the first 16 hex digits of the SHA-256 of the kernel's sources (source_sha);
+# any other sources report traffic as null.
+HEADLINE_SOURCES = ("include/asched.h",) + tuple(
+    "paper_2002_11710_gb300/csrc/" + n for n in ("asched.cu", "full.cu", "kernels.h", "search.cuh", "carry.cuh"))
+TRAFFIC_BYTES = {}
 
 
 def _env_int(k, d):
@@ -91,10 +93,13 @@ def device_ms(fn, reps=5, rounds=3):
     return statistics.median(ts)
 
 
-def source_sha():
-    src = os.path.join(ROOT, "paper_2002_11710_gb300", "csrc", "asched.cu")
-    with open(src, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+def source_sha(root=ROOT):
+    """Of everything the headline kernel is compiled from, and the host code that launches it."""
+    h = hashlib.sha256()
+    for name in HEADLINE_SOURCES:
+        with open(os.path.join(root, name), "rb") as f:
+            h.update(name.encode() + b"\0" + f.read() + b"\0")
+    return h.hexdigest()[:16]
 
 
 def moves_split(M, V):
