@@ -51,3 +51,24 @@ def test_few_small_instances_alone(lo, hi, n):
     _check(_coords("dateline", n, lo, hi), [300.0], "dateline")
     rng = np.random.default_rng(5)
     _check([_points(rng, int(rng.integers(lo, hi + 1)), "plane") for _ in range(n)], [300.0], "plane")
+
+
+@pytest.mark.parametrize("region", ["region", "dateline", "strip", "poles", "close"])
+def test_tiles_at_slow_speeds(region):
+    """At 2 and 10 km/h times run to 10^5 minutes and more, where a float32 error above its screen
+    would show as a wrong integer: half a million pairs each, around the poles and a few hundred
+    metres apart among them."""
+    rng = np.random.default_rng(23)
+    n = 1000
+    if region == "poles":
+        c = np.stack([np.where(rng.random(n) < 0.5, 90.0, -90.0) * (1.0 - 10.0 ** rng.uniform(-9.0, -1.2, n)),
+                      rng.uniform(-180.0, 180.0, n)], axis=1)
+        c[:, 0] = np.abs(c[:, 0])  # one pole: no pair nearly half a turn apart
+    elif region == "close":
+        c = np.stack([rng.uniform(47.0, 47.01, n), rng.uniform(8.0, 8.01, n)], axis=1)
+    elif region == "strip":
+        lon = rng.uniform(176.0, 184.0, n)
+        c = np.stack([rng.uniform(-20.0, -14.0, n), np.where(lon > 180.0, lon - 360.0, lon)], axis=1)
+    else:
+        c = _points(rng, n, region)
+    _check([c, c[:333]], [2.0, 10.0], region)
