@@ -220,10 +220,10 @@ __device__ __forceinline__ Mine load_mine(const CarryCtx& c, int m, int v) {
 constexpr int64_t kNoSwap = INT64_MAX;
 // What the lane's mission reads for node y, all of it for every node (of a route's end too),
 // so that two nodes' loads can go side by side: with 8 or 16 warps an SM a node is a chain of
-// dependent loads. One node at a time, with branches: 1,024 mixed instances 57.8 ms, one of 193
-// missions on 3 vehicles alone 46.2 ms; without branches 56.7 and 40.3; two at a time 52.3 and
-// 38.1 (with a branch around an odd last one, or a loop of its own for short slices, 56 ms:
-// the larger body, and the two evaluations no longer interleaved).
+// dependent loads. One node at a time, with branches: 193 missions on 3 vehicles, alone on 256
+// threads, 46.2 ms for 2,000 iterations; without branches 40.3; two at a time 38.1 (a branch around
+// an odd last one, or a loop of its own for short slices, took it back: the larger body, and the two
+// evaluations no longer interleaved).
 struct NodeTimes {
   int4 x, q, dy;
   int a, b, b2, a3, b3, own, wy;
@@ -503,7 +503,7 @@ __device__ __forceinline__ void carry_solve(const KParams& P, const Layout& lay,
     // 2^lay.ulog of them and at most lay.ucap units. Their lanes take entries' deltas by a
     // 32-bit atomic minimum and leave their keys in pk; the apply step, when the deltas are
     // final, takes the least id among the keys that have it (64-bit shared-memory minima are
-    // compare-and-swap loops: 1.5 us an iteration on the tiny instance).
+    // compare-and-swap loops).
     uint64_t* const pk = reinterpret_cast<uint64_t*>(g_smem + lay.pkey);
     const int vspan = lay.kv * subs;
     const int PV = (V + vspan - 1) / vspan;  // scan units per block
