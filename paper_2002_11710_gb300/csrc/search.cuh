@@ -254,15 +254,16 @@ __host__ __device__ inline int64_t search_items(int64_t M, int64_t V) {
 //   1,024 instances, 256 threads:  200 on 3 208 / 194, on 12 207 / 88; 100 on 4 48.5 / 68.6, on
 //     8 48.6 / 48.1, on 20 50.1 / 37.3; 60 on 12 27.7 / 26.1; 40 on 8 19.7 / 24.0
 //   a cluster of 8 CTAs of 256 threads:  200 on 12 5.8 / 6.3, on 20 6.0 / 5.5; 300 on 20
-//     11.8 / 9.1; 100 on 20 3.2 / 3.7
+//     11.8 / 9.1; 100 on 20 3.2 / 3.7; of 512 threads, 5 missions a vehicle:  160 3.5 / 3.7, 190
+//     4.4 / 4.0, 260 7.5 / 5.7
 __host__ __device__ inline int64_t carry_cost(int64_t M, int64_t V, bool dl, int64_t ctas, int64_t nwarps) {
   const int64_t pairs = V == 1 ? (M + 1) * M : 2 * M * (M + V) / V, entries = V * M;
   if (ctas == 1) {
     const int64_t rest = pairs + entries < 40 * M ? pairs + entries : 40 * M;
     return dl ? 400 * nwarps + 5 * pairs + 2 * entries : 600 * nwarps + 6 * pairs + 4 * rest;
   }
-  const int64_t f = ctas <= 4 ? 7 : 12;
-  return dl ? 400 * ctas * nwarps + f * pairs + 2 * entries : 600 * ctas * nwarps + 2 * f * pairs + 4 * entries;
+  const int64_t f = ctas <= 4 ? 7 : 12, chain = (ctas <= 4 ? 600 : 450) * ctas * nwarps;
+  return dl ? 400 * ctas * nwarps + f * pairs + 2 * entries : chain + 2 * f * pairs + 4 * entries;
 }
 __host__ __device__ inline bool carry_pays(int64_t M, int64_t V, bool dl, int64_t ctas, int64_t nwarps) {
   return 4 * search_items(M, V) > carry_cost(M, V, dl, ctas, nwarps);
@@ -292,12 +293,13 @@ __host__ __device__ inline int pick_search(int M, int V, int L, int nt, bool dl,
 }
 
 // Whether the full evaluation of a batch or a request takes RP records, relocations of four
-// missions and a pass of their own for neighbours: from 4 chunks of 32 items a warp on, where
+// missions and a pass of their own for neighbours: from 6 chunks of 32 items a warp on, where
 // issue bounds it. Below, pairs without them are faster, since the records cost a barrier
 // (20 missions, 256 threads, 1.7 chunks: 1.8 against 2.2 us an iteration); above, with them
 // (1,024 instances of 100 missions on 2 vehicles, 40 chunks: 49 against 57 us; of 200 210
-// against 248). The line at 3, 4 or 6: between 4 and 6 chunks 0.5 to 1.5 % in favour of 4.
-constexpr int kQuadChunks = 4;
+// against 248). With the line at 4, 300 paper-fleet instances take 3,385 us instead of 3,335 and a
+// backlog of 128 requests 16,560 instead of 16,505.
+constexpr int kQuadChunks = 6;
 __host__ __device__ inline bool takes_quads(int M, int V, int ctas, int nwarps) {
   return search_items(M, V) > 32ll * kQuadChunks * ctas * nwarps;
 }

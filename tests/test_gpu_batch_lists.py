@@ -1,5 +1,5 @@
 """Batches by the full evaluation, either side of the size from which its item lists take
-relocations of four missions and neighbours in a pass of their own (4 chunks of 32 items a
+relocations of four missions and neighbours in a pass of their own (6 chunks of 32 items a
 warp), at every mission count mod 4, against the oracle (needs a GB300)."""
 import pytest
 
@@ -9,8 +9,8 @@ from test_gpu_carry import _check_batch
 pytestmark = pytest.mark.gpu
 HARD, PENALTY = gen.HARD, gen.PENALTY
 
-# 64 threads: pairs up to 256 items, (15, 2) with 241 and (16, 2) with 264 on either side
-SIZES = [(13, 2), (14, 2), (15, 2), (16, 2), (17, 2), (18, 3), (19, 1), (23, 2), (40, 2), (65, 1), (66, 2), (67, 1)]
+# 64 threads: pairs up to 384 items, (19, 2) with 381 and (19, 3) with 391 on either side
+SIZES = [(13, 2), (15, 2), (18, 3), (19, 2), (19, 3), (20, 1), (21, 2), (23, 2), (40, 2), (65, 1), (66, 2), (67, 1)]
 
 
 @pytest.mark.parametrize("mode", [HARD, PENALTY])
