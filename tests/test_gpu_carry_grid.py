@@ -72,7 +72,7 @@ EDGES = [(8, 250), (9, 260), (16, 150), (17, 150), (31, 65), (32, 64), (33, 63),
          (97, 30), (150, 5)]
 
 
-@pytest.mark.parametrize("tenure", [0, 1, 7, 60])
+@pytest.mark.parametrize("tenure", [0, 1, 7, 60, 512])
 @pytest.mark.parametrize("compact", [False, True])
 def test_sizes_on_one_cta(tenure, compact):
     insts = [gen.random_instance(300 + 7 * k, n_loc=10 + k, n_vehicles=v, n_missions=m, n_types=2, heli_only_frac=0.2,
